@@ -90,6 +90,16 @@ lat_status derive_model(const lat_params& p, Model* M)
     M->eight_pi_G = p.eight_pi_G;
     M->g8A2 = p.eight_pi_G / (A * A);
     M->inv_sites = 1.0 / ((double)p.n * p.n * p.n);
+    M->grad_scale = M->lap_scale * M->inv_sites;
+    M->sp2 = s + 2.0;
+    M->ch = r * (s - r + 2.0);
+    const double ex[5] = {M->pdom, M->pint, -2.0 * s - 2.0 * r - 1.0, 2.0 * s + 2.0, -2.0 * s - 2.0};
+    int* ei[5] = {&M->e_dom, &M->e_int, &M->e_c, &M->e_v, &M->e_L};
+    M->intpow = 1;
+    for (int k = 0; k < 5; k++) {
+        if (ex[k] == std::rint(ex[k]) && std::fabs(ex[k]) <= 16.0) *ei[k] = (int)ex[k];
+        else M->intpow = 0;
+    }
     return LAT_OK;
 }
 
