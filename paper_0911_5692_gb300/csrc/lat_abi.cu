@@ -242,11 +242,22 @@ lat_status configure_kernel(lat_handle* h, int variant, int ty, int zr, int dept
         return take(cfg, 5);
     }
     if (variant == 0 && h->esize == 4) {
-        // FP32: x tiles one warp wide with compiled geometry where an instance
-        // exists (N = 256, 512, 1024): 512^3 0.871 ms per step against 0.901 ms
-        // (variant 4); 256^3 0.124 against 0.128 ms (variant 2)
+        // FP32: x tiles one warp wide unless they leave too many lanes of the
+        // warp empty. A row of one tile wants 17 lanes (64^3, 16 lanes: 13.1 us per
+        // step against 12.2 of variant 2; 68^3, 17 lanes: 14.4 against 16.5), a
+        // row of several 21 (160^3, 20 lanes: 42.1 against 41.8; 168^3, 21 lanes:
+        // 45.2 against 46.5; 384^3, 32 lanes: 298 against 435). Tiles of 16 rows
+        // with two planes in flight where the lanes are full or the row is one
+        // tile (512^3: 685 us, 8 rows 718; 100^3: 17.7, 17.8), else 8 rows with
+        // three, two blocks to an SM: with empty lanes a block moves fewer bytes
+        // per barrier (200^3: 62 against 64 us, 464^3: 579 against 592, 496^3:
+        // 700 against 710, 704^3: 2050 against 2138).
+        const int q = n / 4, nxt = (q + 31) / 32;
         MarchConfig cfg;
-        if (xw_config(n, 4, 16, 0, 0, &cfg) && fits(cfg)) return take(cfg, 5);
+        if (q / nxt >= (nxt == 1 ? 17 : 21)) {
+            const bool tall = nxt == 1 || q == 32 * nxt;
+            if (xw_config(n, 4, tall ? 16 : 8, 0, tall ? 2 : 3, &cfg) && fits(cfg)) return take(cfg, 5);
+        }
     }
     if (variant == 0 && n / (16 / (int)h->esize) >= 128) {
         // rows of 128 16-byte vectors or more: full-row tiles leave room for at
@@ -298,7 +309,8 @@ std::vector<TuneShape> tune_candidates(const lat_handle* h)
             for (int d : {1, 2}) c.push_back({2, ty, 0, d});
         return c;
     }
-    for (int d : {1, 2}) c.push_back({5, 16, 0, d});
+    for (int d : {1, 2, 3}) c.push_back({5, 16, 0, d});
+    for (int d : {2, 3}) c.push_back({5, 8, 0, d});
     for (int ty : {32, 16, 8})
         for (int d : {1, 2}) c.push_back({4, ty, 0, d});
     for (int ty : {16, 8, 4, 2})

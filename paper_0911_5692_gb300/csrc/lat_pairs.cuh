@@ -32,12 +32,17 @@ __device__ __forceinline__ F2 fma2(F2 a, F2 b, F2 c)
     return r;
 }
 __device__ __forceinline__ D2 mk2(double lo, double hi) { return D2{lo, hi}; }
+__device__ __forceinline__ void un2(D2 a, double& lo, double& hi) { lo = a.x; hi = a.y; }
 __device__ __forceinline__ double lo2(D2 a) { return a.x; }
 __device__ __forceinline__ double hi2(D2 a) { return a.y; }
 __device__ __forceinline__ D2 add2(D2 a, D2 b) { return D2{a.x + b.x, a.y + b.y}; }
 __device__ __forceinline__ D2 sub2(D2 a, D2 b) { return D2{a.x - b.x, a.y - b.y}; }
 __device__ __forceinline__ D2 mul2(D2 a, D2 b) { return D2{a.x * b.x, a.y * b.y}; }
 __device__ __forceinline__ D2 fma2(D2 a, D2 b, D2 c) { return D2{fma(a.x, b.x, c.x), fma(a.y, b.y, c.y)}; }
+
+// scalar subtraction, never contracted: rounds as an element of sub2
+__device__ __forceinline__ float s_sub(float a, float b) { return __fsub_rn(a, b); }
+__device__ __forceinline__ double s_sub(double a, double b) { return __dsub_rn(a, b); }
 
 // A 16-byte vector of one row: NP pairs (4 floats or 2 doubles).
 template <typename T>
@@ -79,5 +84,21 @@ struct PK<double> {
         __stcs(reinterpret_cast<double2*>(p), make_double2(v[0].x, v[0].y));
     }
 };
+
+// x differences of one vector, (right - centre) of each site, given the value
+// right of the last one. The x part of the Laplacian is then the right minus the
+// left difference: (l - c) + (r - c) = (r - c) - (c - l), rounded alike, with
+// every difference formed once (scalar operations that write the halves of the
+// packed pairs: no register moves build shifted pairs).
+template <typename T>
+__device__ __forceinline__ void xdiff(const typename PK<T>::P (&c)[PK<T>::NP], T right, T (&d)[2 * PK<T>::NP])
+{
+    constexpr int VW = 2 * PK<T>::NP;
+    T s[VW];
+#pragma unroll
+    for (int v = 0; v < PK<T>::NP; v++) un2(c[v], s[2 * v], s[2 * v + 1]);
+#pragma unroll
+    for (int i = 0; i < VW; i++) d[i] = s_sub(i + 1 < VW ? s[i + 1] : right, s[i]);
+}
 
 } // namespace lat

@@ -72,11 +72,9 @@ __device__ __forceinline__ void site_kick_drift(const SiteCoefs<T>& C, typename 
 // exactly as the same site in a packed pair (add.rn, mul.rn and fma.rn of the
 // f32x2 instructions act per element).
 __device__ __forceinline__ float s_add(float a, float b) { return __fadd_rn(a, b); }
-__device__ __forceinline__ float s_sub(float a, float b) { return __fsub_rn(a, b); }
 __device__ __forceinline__ float s_mul(float a, float b) { return __fmul_rn(a, b); }
 __device__ __forceinline__ float s_fma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 __device__ __forceinline__ double s_add(double a, double b) { return __dadd_rn(a, b); }
-__device__ __forceinline__ double s_sub(double a, double b) { return __dsub_rn(a, b); }
 __device__ __forceinline__ double s_mul(double a, double b) { return __dmul_rn(a, b); }
 __device__ __forceinline__ double s_fma(double a, double b, double c) { return __fma_rn(a, b, c); }
 

@@ -15,8 +15,8 @@ const void* slab_xw_fn(int n, size_t* smem, int* depth)
 #define LAT_SLAB_XW_CASE(NN, DD)                                              \
     if (n == NN) {                                                            \
         *depth = DD;                                                          \
-        *smem = xw::XW<T, NN, 16, DD, true>::SMEM;                            \
-        return (const void*)xw::step_xw_kernel<T, NN, 16, DD, true>;          \
+        *smem = xw::XW<T, 16, DD, true>::SMEM;                            \
+        return (const void*)xw::step_xw_kernel<T, 16, DD, true>;          \
     }
     // two planes in flight for FP32 (as the whole-lattice default), one for FP64
     if constexpr (sizeof(T) == 4) {
@@ -39,7 +39,7 @@ bool slab_xw_config(int n, int elem_bytes, int nz, MarchConfig* cfg)
     if (!fn || smem > 227 * 1024 - 2048) return false;
     constexpr int ty = 16;
     const int vw = 16 / elem_bytes, w = 32 * vw, nxt = n / w;
-    const int threads = (ty + 4) * 32;
+    const int threads = (ty / 2 + 2) * 32;
     if (allow_dynamic_smem(fn, smem) != cudaSuccess) return false;
     int occ = 0, dev = 0, sms = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, threads, smem) != cudaSuccess || occ < 1) return false;

@@ -9,37 +9,25 @@ namespace lat {
 
 namespace {
 
-// Compiled instances: (element bytes, N, TY, D).
-struct XWKey {
-    int esize, n, ty, depth;
-};
-constexpr XWKey kXW[] = {{4, 256, 16, 1}, {4, 256, 16, 2}, {4, 512, 16, 1}, {4, 512, 16, 2}, {4, 1024, 16, 1},
-                         {8, 256, 16, 1}, {8, 512, 16, 1}};
-
+// The compiled instance of a tile height and prefetch depth, or null.
 template <typename T>
-const void* xw_fn(int n, int ty, int depth, size_t* smem)
+const void* xw_fn(int ty, int depth, size_t* smem)
 {
-#define LAT_XW_CASE(NN, TT, DD)                                  \
-    if (n == NN && ty == TT && depth == DD) {                    \
-        *smem = xw::XW<T, NN, TT, DD, false>::SMEM;              \
-        return (const void*)xw::step_xw_kernel<T, NN, TT, DD, false>; \
+#define LAT_XW_CASE(TT, DD)                                 \
+    if (ty == TT && depth == DD) {                          \
+        *smem = xw::XW<T, TT, DD, false>::SMEM;             \
+        return (const void*)xw::step_xw_kernel<T, TT, DD, false>; \
     }
-    if constexpr (sizeof(T) == 4) {
-        LAT_XW_CASE(256, 16, 1) LAT_XW_CASE(256, 16, 2) LAT_XW_CASE(512, 16, 1) LAT_XW_CASE(512, 16, 2)
-        LAT_XW_CASE(1024, 16, 1)
-    } else {
-        LAT_XW_CASE(256, 16, 1) LAT_XW_CASE(512, 16, 1)
-    }
+    LAT_XW_CASE(16, 1) LAT_XW_CASE(16, 2)
+    if constexpr (sizeof(T) == 4) { LAT_XW_CASE(16, 3) LAT_XW_CASE(8, 2) LAT_XW_CASE(8, 3) }
+    else { LAT_XW_CASE(8, 1) LAT_XW_CASE(4, 1) }
 #undef LAT_XW_CASE
     return nullptr;
 }
 
-const void* xw_kernel(int esize, int n, int ty, int depth, size_t* smem)
+const void* xw_kernel(int esize, int ty, int depth, size_t* smem)
 {
-    for (const XWKey& k : kXW)
-        if (k.esize == esize && k.n == n && k.ty == ty && k.depth == depth)
-            return esize == 4 ? xw_fn<float>(n, ty, depth, smem) : xw_fn<double>(n, ty, depth, smem);
-    return nullptr;
+    return esize == 4 ? xw_fn<float>(ty, depth, smem) : xw_fn<double>(ty, depth, smem);
 }
 
 } // namespace
@@ -47,29 +35,29 @@ const void* xw_kernel(int esize, int n, int ty, int depth, size_t* smem)
 bool xw_config(int n, int elem_bytes, int ty, int zr, int depth, MarchConfig* cfg)
 {
     const int tyv = ty > 0 ? ty : 16;
-    // the instance with the requested depth, else any compiled depth (2 first:
-    // two planes in flight measured 0.811-0.816 against 0.860 ms per step at
-    // 512^3 FP32, 0.117 against 0.124 ms at 256^3)
+    // the instance with the requested depth, else any compiled depth (2 first: a
+    // second plane in flight takes the 512^3 FP32 step from 843 to 685 us and the
+    // 256^3 step from 114 to 98; a third changes them by less than the runs differ)
     int d = depth;
     size_t smem = 0;
     const void* fn = nullptr;
-    if (d > 0) fn = xw_kernel(elem_bytes, n, tyv, d, &smem);
+    if (d > 0) fn = xw_kernel(elem_bytes, tyv, d, &smem);
     else
         for (int dd : {2, 1})
-            if ((fn = xw_kernel(elem_bytes, n, tyv, dd, &smem))) {
+            if ((fn = xw_kernel(elem_bytes, tyv, dd, &smem))) {
                 d = dd;
                 break;
             }
     if (!fn || smem > 227 * 1024 - 2048) return false;
-    const int vw = 16 / elem_bytes, w = 32 * vw, nxt = n / w;
-    const int threads = (tyv + 4) * 32;
+    const int vw = 16 / elem_bytes, nxt = (n / vw + 31) / 32;
+    const int threads = (tyv / 2 + 2) * 32;
     if (allow_dynamic_smem(fn, smem) != cudaSuccess) return false;
     int occ = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, threads, smem) != cudaSuccess || occ < 1) return false;
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) return false;
-    const int nyt = n / tyv;
+    const int nyt = (n + tyv - 1) / tyv;
     const long long tiles = (long long)nyt * nxt, units = tiles * n;
     long long blocks = 0;
     // whole groups of nxt blocks (the x tiles of a y tile, marching together)
@@ -103,7 +91,7 @@ cudaError_t launch_step_xw(const Bufs<T>& b, const Model& M, DevScalars* sc, dou
                            cudaStream_t st)
 {
     size_t smem = 0;
-    const void* fn = xw_fn<T>(M.n, cfg.ty, cfg.depth, &smem);
+    const void* fn = xw_fn<T>(cfg.ty, cfg.depth, &smem);
     if (!fn) return cudaErrorInvalidValue;
     xw::SlabRun R{0, 0, nullptr};
     void* args[] = {(void*)&b, (void*)&M, (void*)&sc, (void*)&partials, (void*)&R};
