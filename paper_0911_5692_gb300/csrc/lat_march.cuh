@@ -160,6 +160,11 @@ __device__ void march_segment(const MarchLattice<T>& L, int yt, int z0, int nz, 
         cp_async_commit();
     }
     int sf = 0, sp = 0;          // k mod (D+3), k mod (D+1)
+    // centre minus the plane below. The FP64 step, bound by its FP64 operations,
+    // keeps it from the plane before (128^3: 262 -> 254 us); in FP32 the carried
+    // registers cost more than the shared load (64^3: 12.15 -> 12.3 us).
+    constexpr bool kShare = sizeof(T) == 8;
+    P dzp[2][NP];
 
     for (int k = 0; k <= nz; k++) {
         const bool ahead = k == nz;
@@ -200,34 +205,32 @@ __device__ void march_segment(const MarchLattice<T>& L, int yt, int z0, int nz, 
 #pragma unroll
             for (int f = 0; f < 2; f++) {
                 const T* Ff = Fc + f * R.fieldF + offF;
-                P up[NP], dn[NP], zm[NP], zp[NP], pv[NP], lft[NP], rgt[NP];
+                P up[NP], dn[NP], zp[NP], pv[NP];
                 PK<T>::ld(Ff - n, up);
                 PK<T>::ld(Ff + n, dn);
-                PK<T>::ld(Fm + f * R.fieldF + offF, zm);
+                if (!kShare || k == 0) {
+                    P zm[NP];
+                    PK<T>::ld(Fm + f * R.fieldF + offF, zm);
+#pragma unroll
+                    for (int v = 0; v < NP; v++) dzp[f][v] = sub2(cen[f][v], zm[v]);
+                }
                 PK<T>::ld(Fp + f * R.fieldF + offF, zp);
                 PK<T>::ld(Pc + f * R.fieldP + offP, pv);
-                const T left = lefts[f], right = rights[f];
-                if constexpr (NP == 2) {
-                    T c0, c1, c2, c3;
-                    un2(cen[f][0], c0, c1);
-                    un2(cen[f][1], c2, c3);
-                    lft[0] = mk2(left, c0);
-                    lft[1] = mk2(c1, c2);
-                    rgt[0] = lft[1];
-                    rgt[1] = mk2(c3, right);
-                } else {
-                    lft[0] = mk2(left, lo2(cen[f][0]));
-                    rgt[0] = mk2(hi2(cen[f][0]), right);
-                }
+                T d[VW];
+                xdiff<T>(cen[f], rights[f], d);
+                const T dl = s_sub(lo2(cen[f][0]), lefts[f]);
                 const P dtcl2 = mk2(L.K.dtcl, L.K.dtcl), dtcf2 = mk2(L.K.dtcf, L.K.dtcf);
 #pragma unroll
                 for (int v = 0; v < NP; v++) {
                     const P c = cen[f][v];
-                    // Laplacian as a sum of neighbour differences: exact differences
-                    // for f = const + small (Sterbenz)
-                    const P lapu = add2(add2(add2(sub2(lft[v], c), sub2(rgt[v], c)),
-                                             add2(sub2(up[v], c), sub2(dn[v], c))),
-                                        add2(sub2(zm[v], c), sub2(zp[v], c)));
+                    // Laplacian as a sum of neighbour differences, exact for f =
+                    // const + small (Sterbenz); the x differences serve both
+                    // sites beside them, the z difference this plane and the next
+                    // ((zm - c) + (zp - c) = (zp - c) - (c - zm), rounded alike)
+                    const P lx = mk2(s_sub(d[2 * v], v == 0 ? dl : d[2 * v - 1]), s_sub(d[2 * v + 1], d[2 * v]));
+                    const P dz = sub2(zp[v], c);
+                    const P lapu = add2(add2(lx, add2(sub2(up[v], c), sub2(dn[v], c))), sub2(dz, dzp[f][v]));
+                    dzp[f][v] = dz;
                     pn[f][v] = fma2(dtcl2, lapu, fma2(dtcf2, c, pv[v]));
                 }
             }
@@ -266,22 +269,14 @@ __device__ void march_segment(const MarchLattice<T>& L, int yt, int z0, int nz, 
 #pragma unroll
             for (int f = 0; f < 2; f++) {
                 const T* Gf = Gr + f * R.fieldG + offP;
-                P yn[NP], xn[NP];
+                P yn[NP];
                 PK<T>::ld(Gf + n, yn);
-                const T xnext = xnexts[f];
-                if constexpr (NP == 2) {
-                    T a, b, c, d;
-                    un2(gq[f][0], a, b);
-                    un2(gq[f][1], c, d);
-                    xn[0] = mk2(b, c);
-                    xn[1] = mk2(d, xnext);
-                } else {
-                    xn[0] = mk2(hi2(gq[f][0]), xnext);
-                }
+                T d[VW];
+                xdiff<T>(gq[f], xnexts[f], d);
                 P acc = f == 0 ? A.accg0 : A.accg1;
 #pragma unroll
                 for (int v = 0; v < NP; v++) {
-                    const P dxv = sub2(xn[v], gq[f][v]), dyv = sub2(yn[v], gq[f][v]), dzv = sub2(g[f][v], gq[f][v]);
+                    const P dxv = mk2(d[2 * v], d[2 * v + 1]), dyv = sub2(yn[v], gq[f][v]), dzv = sub2(g[f][v], gq[f][v]);
                     acc = fma2(dxv, dxv, fma2(dyv, dyv, fma2(dzv, dzv, acc)));
                 }
                 if (f == 0) A.accg0 = acc;

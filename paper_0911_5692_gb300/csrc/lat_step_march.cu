@@ -224,10 +224,52 @@ bool march_slab_config(int n, int elem_bytes, int nzl, MarchConfig* cfg)
     return false;
 }
 
+// FP64 tiles and blocks. The step is bound by the FP64 pipes, one per SM sub-
+// partition, 64 cycles per warp instruction: about 32 instructions per two sites
+// that a thread kicks and 16 for the sums of two it owns. A block of ty rows and
+// P planes kicks (ty + 1)(P + 1) rows for its ty P, so tall tiles and long runs
+// cost least, but the busiest sub-partition decides: the tile height and block
+// count are those with the least time there, each plane step costing about 5000
+// cycles (its chain of dependent operations) beside its instructions. 32^3: 64
+// blocks of a plane of 16 rows 24.3 us per step, 128 of 8 rows 17.5; 96^3 150 ->
+// 124; 72^3 88 -> 67; 56^3 55 -> 48.
+bool march_config_fp64(int n, int depth, MarchConfig* cfg)
+{
+    bool found = false;
+    double best = 0.0;
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) return false;
+    for (int ty : {16, 8, 4, 2, 1}) {
+        MarchConfig c;
+        if (!march_geom(n, 8, ty, 0, depth, &c)) continue;
+        const long long units = (long long)c.nyt * n, most = c.blocks;
+        for (int k = 1; k * sms <= std::max<long long>(most, sms); k++) {   // blocks per SM
+            const long long slots = std::min<long long>((long long)k * sms, units);
+            const long long P = (units + slots - 1) / slots, blocks = P >= 8 ? slots : (units + P - 1) / P;
+            const long long per_sm = (blocks + sms - 1) / sms;
+            // warps on the busiest sub-partition (two sites per lane)
+            const double warps = (double)((per_sm * (ty + 1) * (n / 2) + 127) / 128);
+            const double planes = P >= 8 ? (double)units / blocks : (double)P;   // per block
+            const double cost = warps * 128.0 * (32.0 * (planes + 1) + 16.0 * planes) +
+                                5000.0 * per_sm * (planes + 1);
+            if (blocks > most || (found && cost >= best)) continue;
+            found = true;
+            best = cost;
+            *cfg = c;
+            cfg->blocks = (int)blocks;
+            cfg->zr = (int)P;
+            cfg->nzc = (int)((blocks + c.nyt - 1) / c.nyt);
+        }
+    }
+    return found;
+}
+
 bool march_config(int n, int elem_bytes, int ty, int zr, int depth, MarchConfig* cfg)
 {
     const int d = depth > 0 ? depth : 1;
     if (ty > 0) return march_geom(n, elem_bytes, ty, zr, d, cfg);
+    if (elem_bytes == 8 && zr == 0) return march_config_fp64(n, d, cfg);
     const int tys[] = {16, 8, 4, 2, 1};
     for (int t : tys)
         if (march_geom(n, elem_bytes, t, zr, d, cfg)) return true;
