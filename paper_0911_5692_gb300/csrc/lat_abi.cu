@@ -156,19 +156,24 @@ lat_status launch_prepare(lat_handle* h)
 }
 
 // One step of the configured kernel on the given buffers (the handle's own for
-// lat_evolve; per-step storage for the recomputation of the reverse pass).
+// lat_evolve; per-step storage for the recomputation of the reverse pass);
+// `chain`: the stream's last work is a step kernel of the same call.
 template <typename T>
-cudaError_t launch_step_with(lat_handle* h, const Bufs<T>& b, bool)
+cudaError_t launch_step_with(lat_handle* h, const Bufs<T>& b, bool chain)
 {
-    return launch_step_march<T>(b, h->M, h->sc, h->partials, h->mcfg, h->stream);
+    MarchConfig cfg = h->mcfg;
+    // not behind the L = 1/H form's pass: its blocks, set up beside the step's, keep
+    // the step's shared-memory split of L1 (256^3: 202 us per step chained, 198 not)
+    cfg.chain = chain && h->M.expansion != 2;
+    return launch_step_march<T>(b, h->M, h->sc, h->partials, cfg, h->stream);
 }
 template cudaError_t launch_step_with<float>(lat_handle*, const Bufs<float>&, bool);
 template cudaError_t launch_step_with<double>(lat_handle*, const Bufs<double>&, bool);
 
-lat_status launch_one_step(lat_handle* h)
+lat_status launch_one_step(lat_handle* h, bool chain)
 {
-    cudaError_t e = h->prec == 32 ? launch_step_with<float>(h, bufs_of<float>(h), true)
-                                  : launch_step_with<double>(h, bufs_of<double>(h), true);
+    cudaError_t e = h->prec == 32 ? launch_step_with<float>(h, bufs_of<float>(h), chain)
+                                  : launch_step_with<double>(h, bufs_of<double>(h), chain);
     LAT_TRY(cuda_status(e));
     return launch_lform_pass(h);
 }
@@ -577,7 +582,7 @@ lat_status lat_evolve(lat_handle* h, int64_t n_steps)
             cudaGraph_t g;
             LAT_CUDA(cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal));
             lat_status st = LAT_OK;
-            for (int i = 0; i < kGraphChunk && st == LAT_OK; i++) st = launch_one_step(h);
+            for (int i = 0; i < kGraphChunk && st == LAT_OK; i++) st = launch_one_step(h, i > 0);
             cudaError_t e = cudaStreamEndCapture(h->stream, &g);
             if (st != LAT_OK) return st;
             if (e != cudaSuccess) return LAT_ECUDA;
@@ -591,7 +596,7 @@ lat_status lat_evolve(lat_handle* h, int64_t n_steps)
             left -= h->graph_steps;
         }
     }
-    for (; left > 0; left--) LAT_TRY(launch_one_step(h));
+    for (bool chain = false; left > 0; left--, chain = true) LAT_TRY(launch_one_step(h, chain));
     return LAT_OK;
 }
 
@@ -812,7 +817,7 @@ lat_status lat_evolve_host(lat_handle* h, void* const host[4], int64_t n_steps, 
         if (st != LAT_OK) break;
         // the step: the sums of the uploaded fields, then the fused step
         h->dirty = true;
-        if ((st = ensure_prepared(h)) != LAT_OK || (st = launch_one_step(h)) != LAT_OK) break;
+        if ((st = ensure_prepared(h)) != LAT_OK || (st = launch_one_step(h, false)) != LAT_OK) break;
         if (dlog) ok(cudaMemcpyAsync(dlog + k, h->sc, sizeof(DevScalars), cudaMemcpyDeviceToDevice, h->stream));
         ok(cudaEventRecord(comp_done, h->stream)) && ok(cudaStreamWaitEvent(down, comp_done, 0));
         // down: the evolved set, chunk by chunk

@@ -981,7 +981,7 @@ lat_status vjp_impl(lat_handle* h, int64_t n, int64_t ckpt_every, T* fb_user, T*
             }
             LAT_CUDA(cudaMemcpyAsync(ck_sc + k / K, h->sc, sizeof(DevScalars), cudaMemcpyDeviceToDevice, st));
         }
-        LAT_CUDA(launch_step_with<T>(h, hb, false));
+        LAT_CUDA(launch_step_with<T>(h, hb, k % K != 0));
     }
     LAT_TRY(guard.clear());
     const int parN = (int)((s0.step + n) & 1);
@@ -1094,7 +1094,7 @@ lat_status vjp_impl(lat_handle* h, int64_t n, int64_t ckpt_every, T* fb_user, T*
                 b.f[par][f] = arr(seg, (size_t)(k - c) * 2 + f);
                 b.f[1 - par][f] = arr(seg, (size_t)(k - c + 1) * 2 + f);
             }
-            LAT_CUDA(launch_step_with<T>(h, b, false));
+            LAT_CUDA(launch_step_with<T>(h, b, k > c));
         }
         // reverse steps e-1 .. c
         for (int64_t k = e - 1; k >= c; k--) {

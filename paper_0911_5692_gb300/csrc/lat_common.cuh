@@ -180,6 +180,17 @@ __device__ __forceinline__ void block_reduce(double v[kSums], double* red, doubl
     for (int k = 0; k < kSums; k++) out[k] = v[k];
 }
 
+// The start of a kernel launched by launch_chained: everything the kernels before
+// it wrote is visible after this, and the kernel after it may now be set up on
+// the SMs that this one leaves. Nothing the stream's earlier work writes is read
+// before it; what needs the launch arguments alone (the tile geometry) goes
+// before.
+__device__ __forceinline__ void chain_begin()
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 // a^p. The exponents of the two models' rescalings (Sec. II.B) are integers
 // for which repeated multiplication of a (or of inv_a = 1/a for negative p) is
 // exact to a few ulp and costs a handful of FP64 multiplies instead of a

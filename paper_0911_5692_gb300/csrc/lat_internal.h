@@ -68,6 +68,6 @@ lat_status ensure_prepared(lat_handle* h);
 lat_status read_scalars(lat_handle* h, DevScalars* out);
 void drop_graph(lat_handle* h);
 template <typename T>
-cudaError_t launch_step_with(lat_handle* h, const Bufs<T>& b, bool own_buffers);
+cudaError_t launch_step_with(lat_handle* h, const Bufs<T>& b, bool chain);
 
 } // namespace lat

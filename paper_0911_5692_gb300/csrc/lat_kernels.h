@@ -31,6 +31,17 @@ cudaError_t launch_sums(const Bufs<T>& b, const Model& M, DevScalars* sc, double
 // lower limit set for one would refuse the launches of another.
 cudaError_t allow_dynamic_smem(const void* fn, size_t bytes);
 
+// Launch a kernel that begins with chain_begin() (lat_common.cuh) so that its
+// blocks are set up while the kernel before it on the stream drains (programmatic
+// stream serialisation, also as edges of a captured graph): 1.47 -> 1.05 us from
+// one empty kernel to the next in a graph, 4.1 -> 1.4 us outside one, and the tile
+// geometry is formed meanwhile. Only where `chain` says that the stream's last
+// work is a kernel this library launched in the same call (nothing of the
+// caller's, no copy and no wait for an event lies between); else, and on the
+// legacy default stream, a plain launch.
+cudaError_t launch_chained(const void* fn, dim3 grid, dim3 block, void** args, size_t smem, cudaStream_t st,
+                           bool chain);
+
 struct MarchConfig {
     int ty;        // owned rows per tile
     int zr;        // planes per z-chunk (the longest)
@@ -47,6 +58,7 @@ struct MarchConfig {
     int s27 = 0;   // 1: the 27-point Laplacian kernel (lat_step27.cu)
     int nxt = 1;   // 27-point and x-tiled kernels: x tiles per row
     int xt = 0;    // 1: the x-tiled 7-point kernel (lat_step_xt.cu)
+    int chain = 0; // 1: launched behind a kernel of the same call (launch_chained)
     int xw = 0;    // 1: the compile-time x-tiled kernel one warp wide (lat_step_xw.cu)
 };
 // kernel specialised for (element bytes, N, ty, depth), or null; *smem gets its

@@ -387,6 +387,7 @@ __global__ void __launch_bounds__(MAXT, 1) step27_kernel(Bufs<T> B, Model M, Dev
 {
     __shared__ double red[32 * kSums];
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    chain_begin();
     if (sc->status != LAT_OK) return;
     T* const S = reinterpret_cast<T*>(smem_raw);
     const int n = M.n;
@@ -539,13 +540,15 @@ cudaError_t launch_step27(const Bufs<T>& b, const Model& M, DevScalars* sc, doub
                           cudaStream_t st)
 {
     Args27 G{cfg.ty, cfg.nyt, cfg.depth, cfg.nxt, M.n / cfg.nxt};
+    const void* fn;
     switch (cfg.maxt) {
-    case 256: step27_kernel<T, 256><<<cfg.blocks, cfg.threads, cfg.smem, st>>>(b, M, sc, partials, G); break;
-    case 512: step27_kernel<T, 512><<<cfg.blocks, cfg.threads, cfg.smem, st>>>(b, M, sc, partials, G); break;
-    case 768: step27_kernel<T, 768><<<cfg.blocks, cfg.threads, cfg.smem, st>>>(b, M, sc, partials, G); break;
-    default: step27_kernel<T, 1024><<<cfg.blocks, cfg.threads, cfg.smem, st>>>(b, M, sc, partials, G); break;
+    case 256: fn = (const void*)step27_kernel<T, 256>; break;
+    case 512: fn = (const void*)step27_kernel<T, 512>; break;
+    case 768: fn = (const void*)step27_kernel<T, 768>; break;
+    default: fn = (const void*)step27_kernel<T, 1024>; break;
     }
-    return cudaGetLastError();
+    void* args[] = {(void*)&b, (void*)&M, (void*)&sc, (void*)&partials, (void*)&G};
+    return launch_chained(fn, dim3(cfg.blocks), dim3(cfg.threads), args, cfg.smem, st, cfg.chain);
 }
 
 template cudaError_t launch_step27<float>(const Bufs<float>&, const Model&, DevScalars*, double*, const MarchConfig&,

@@ -476,6 +476,7 @@ __global__ void __launch_bounds__(S27<T, N, TY, D>::THREADS, 1)
     constexpr int VW = F::VW, W = F::W, NXT = F::NXT;
     __shared__ double red[32 * kSums];
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    chain_begin();
     if (sc->status != LAT_OK) return;
 
     typename F::Ctx C;
@@ -619,7 +620,7 @@ cudaError_t launch_step27w(const Bufs<T>& b, const Model& M, DevScalars* sc, dou
     const void* fn = s27w_fn<T>(M.n, cfg.ty, cfg.depth, &smem);
     if (!fn) return cudaErrorInvalidValue;
     void* args[] = {(void*)&b, (void*)&M, (void*)&sc, (void*)&partials};
-    return cudaLaunchKernel(fn, dim3(cfg.blocks), dim3(cfg.threads), args, cfg.smem, st);
+    return launch_chained(fn, dim3(cfg.blocks), dim3(cfg.threads), args, cfg.smem, st, cfg.chain);
 }
 
 template cudaError_t launch_step27w<float>(const Bufs<float>&, const Model&, DevScalars*, double*, const MarchConfig&,

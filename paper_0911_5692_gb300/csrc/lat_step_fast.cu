@@ -210,6 +210,7 @@ __global__ void __launch_bounds__(Fast<T, N, TY, D>::THREADS, (Fast<T, N, TY, D>
     constexpr int VW = F::VW;
     __shared__ double red[32 * kSums];
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    chain_begin();
     if (sc->status != LAT_OK) return;
 
     typename F::Ctx C;
@@ -325,7 +326,7 @@ cudaError_t launch_step_fast(const Bufs<T>& b, const Model& M, DevScalars* sc, d
     const void* fn = fast_fn<T>(M.n, cfg.ty, cfg.depth, &smem);
     if (!fn) return cudaErrorInvalidValue;
     void* args[] = {(void*)&b, (void*)&M, (void*)&sc, (void*)&partials};
-    return cudaLaunchKernel(fn, dim3(cfg.blocks), dim3(cfg.threads), args, cfg.smem, st);
+    return launch_chained(fn, dim3(cfg.blocks), dim3(cfg.threads), args, cfg.smem, st, cfg.chain);
 }
 
 template cudaError_t launch_step_fast<float>(const Bufs<float>&, const Model&, DevScalars*, double*,

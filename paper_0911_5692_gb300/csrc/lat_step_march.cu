@@ -37,6 +37,21 @@ cudaError_t allow_dynamic_smem(const void* fn, size_t bytes)
     return e;
 }
 
+cudaError_t launch_chained(const void* fn, dim3 grid, dim3 block, void** args, size_t smem, cudaStream_t st, bool chain)
+{
+    if (st == nullptr || !chain) return cudaLaunchKernel(fn, grid, block, args, smem, st);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelExC(&cfg, fn, args);
+}
 
 namespace {
 
@@ -53,6 +68,7 @@ __global__ void __launch_bounds__(MAXT, (MAXT <= 512 ? 2 : 1))
 {
     __shared__ double red[32 * kSums];
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    chain_begin();
     if (sc->status != LAT_OK) return;
     T* const S = reinterpret_cast<T*>(smem_raw);
     const int n = M.n;
@@ -297,7 +313,7 @@ cudaError_t launch_step_march(const Bufs<T>& b, const Model& M, DevScalars* sc, 
     double* so = sums_out;
     const void* fn = march_fn<T>(cfg.maxt, M.split != 0);
     void* args[] = {(void*)&b, (void*)&M, (void*)&sc, (void*)&partials, (void*)&G, (void*)&so};
-    cudaError_t e = cudaLaunchKernel(fn, dim3(cfg.blocks), dim3(cfg.threads), args, cfg.smem, st);
+    cudaError_t e = launch_chained(fn, dim3(cfg.blocks), dim3(cfg.threads), args, cfg.smem, st, cfg.chain && !sums_out);
     if (e != cudaSuccess) return e;
     return cudaGetLastError();
 }

@@ -226,6 +226,7 @@ __global__ void __launch_bounds__(MAXT, 1) step_xt_kernel(Bufs<T> B, Model M, De
 {
     __shared__ double red[32 * kSums];
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    chain_begin();
     if (sc->status != LAT_OK) return;
     T* const S = reinterpret_cast<T*>(smem_raw);
     const int n = M.n;
@@ -372,14 +373,16 @@ cudaError_t launch_step_xt(const Bufs<T>& b, const Model& M, DevScalars* sc, dou
                            cudaStream_t st)
 {
     ArgsXt G{cfg.ty, cfg.nyt, cfg.depth, cfg.nxt, M.n / cfg.nxt};
+    const void* fn;
     switch (cfg.maxt) {
-    case 384: step_xt_kernel<T, 384><<<cfg.blocks, cfg.threads, cfg.smem, st>>>(b, M, sc, partials, G); break;
-    case 512: step_xt_kernel<T, 512><<<cfg.blocks, cfg.threads, cfg.smem, st>>>(b, M, sc, partials, G); break;
-    case 640: step_xt_kernel<T, 640><<<cfg.blocks, cfg.threads, cfg.smem, st>>>(b, M, sc, partials, G); break;
-    case 768: step_xt_kernel<T, 768><<<cfg.blocks, cfg.threads, cfg.smem, st>>>(b, M, sc, partials, G); break;
-    default: step_xt_kernel<T, 1024><<<cfg.blocks, cfg.threads, cfg.smem, st>>>(b, M, sc, partials, G); break;
+    case 384: fn = (const void*)step_xt_kernel<T, 384>; break;
+    case 512: fn = (const void*)step_xt_kernel<T, 512>; break;
+    case 640: fn = (const void*)step_xt_kernel<T, 640>; break;
+    case 768: fn = (const void*)step_xt_kernel<T, 768>; break;
+    default: fn = (const void*)step_xt_kernel<T, 1024>; break;
     }
-    return cudaGetLastError();
+    void* args[] = {(void*)&b, (void*)&M, (void*)&sc, (void*)&partials, (void*)&G};
+    return launch_chained(fn, dim3(cfg.blocks), dim3(cfg.threads), args, cfg.smem, st, cfg.chain);
 }
 
 template cudaError_t launch_step_xt<float>(const Bufs<float>&, const Model&, DevScalars*, double*, const MarchConfig&,

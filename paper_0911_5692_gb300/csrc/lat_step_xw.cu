@@ -95,7 +95,7 @@ cudaError_t launch_step_xw(const Bufs<T>& b, const Model& M, DevScalars* sc, dou
     if (!fn) return cudaErrorInvalidValue;
     xw::SlabRun R{0, 0, nullptr};
     void* args[] = {(void*)&b, (void*)&M, (void*)&sc, (void*)&partials, (void*)&R};
-    return cudaLaunchKernel(fn, dim3(cfg.blocks), dim3(cfg.threads), args, cfg.smem, st);
+    return launch_chained(fn, dim3(cfg.blocks), dim3(cfg.threads), args, cfg.smem, st, cfg.chain);
 }
 
 template cudaError_t launch_step_xw<float>(const Bufs<float>&, const Model&, DevScalars*, double*, const MarchConfig&,

@@ -449,28 +449,10 @@ __global__ void __launch_bounds__(XW<T, TY, D, SLAB>::THREADS, TY <= 8 ? 2 : 1)
     constexpr int VW = F::VW, W = F::W;
     __shared__ double red[32 * kSums];
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    if (sc->status != LAT_OK) return;
-
     typename F::Ctx C;
     C.S = reinterpret_cast<T*>(smem_raw);
     const int warp = threadIdx.x >> 5;
     C.lane = threadIdx.x & 31;
-    const bool par = (sc->step & 1) != 0;
-    if constexpr (!SLAB) {
-        C.f0 = par ? B.f[1][0] : B.f[0][0];
-        C.f1 = par ? B.f[1][1] : B.f[0][1];
-        C.p0 = par ? B.p[1][0] : B.p[0][0];
-        C.p1 = par ? B.p[1][1] : B.p[0][1];
-        C.of0 = par ? B.f[0][0] : B.f[1][0];
-        C.of1 = par ? B.f[0][1] : B.f[1][1];
-        C.op0 = par ? B.p[0][0] : B.p[1][0];
-        C.op1 = par ? B.p[0][1] : B.p[1][1];
-    }
-    C.K = site_coefs<T>(sc, M.beta);
-    C.dtcl2 = mk2(C.K.dtcl, C.K.dtcl);
-    C.dtcf2 = mk2(C.K.dtcf, C.K.dtcf);
-    typename F::Acc A;
-    A.zero();
 
     // groups of nxt blocks: the x tiles of one y tile, marching the same
     // (y tile, z plane) units
@@ -494,6 +476,26 @@ __global__ void __launch_bounds__(XW<T, TY, D, SLAB>::THREADS, TY <= 8 ? 2 : 1)
     C.exl = (uint32_t)(x0 == 0 ? n - 1 : x0 - 1);
     C.exr = (uint32_t)(x1 == n ? 0 : x1);
     C.exr1 = (uint32_t)(x1 + 1 >= n ? x1 + 1 - n : x1 + 1);
+
+    chain_begin();
+    if (sc->status != LAT_OK) return;
+    const bool par = (sc->step & 1) != 0;
+    if constexpr (!SLAB) {
+        C.f0 = par ? B.f[1][0] : B.f[0][0];
+        C.f1 = par ? B.f[1][1] : B.f[0][1];
+        C.p0 = par ? B.p[1][0] : B.p[0][0];
+        C.p1 = par ? B.p[1][1] : B.p[0][1];
+        C.of0 = par ? B.f[0][0] : B.f[1][0];
+        C.of1 = par ? B.f[0][1] : B.f[1][1];
+        C.op0 = par ? B.p[0][0] : B.p[1][0];
+        C.op1 = par ? B.p[0][1] : B.p[1][1];
+    }
+    C.K = site_coefs<T>(sc, M.beta);
+    C.dtcl2 = mk2(C.K.dtcl, C.K.dtcl);
+    C.dtcf2 = mk2(C.K.dtcf, C.K.dtcf);
+    typename F::Acc A;
+    A.zero();
+
     C.zb = 0;
     int yt;
     for (bool first = true; walk.run(yt, C.z0, C.nz); first = false) {
