@@ -388,7 +388,7 @@ lat_status lat_set_g2(lat_handle* h, double g2);
  *   ckpt_every: steps between stored checkpoints; 0 = ceil(sqrt(n_steps)). The
  *     forward pass stores one checkpoint (three field pairs) per ckpt_every
  *     steps, the reverse pass recomputes each segment into ckpt_every field
- *     pairs; device memory grows as (3 n_steps / ckpt_every + 2 ckpt_every + 8)
+ *     pairs; device memory grows as (6 n_steps / ckpt_every + 2 ckpt_every + 10)
  *     arrays.
  * The handle ends at the state after n_steps (as after lat_evolve).
  * Synchronises. LAT_ENOMEM if the checkpoints do not fit; LAT_EUNSUPPORTED for

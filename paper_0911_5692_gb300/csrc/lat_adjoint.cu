@@ -23,6 +23,7 @@
 #include <cstddef>
 #include <cstring>
 #include <type_traits>
+#include <utility>
 #include <vector>
 
 #include "lat_async.cuh"
@@ -35,13 +36,39 @@ namespace {
 
 constexpr int kAdjThreads = 256;
 
-// Adjoint scalars carried between reverse steps (FP64, device).
+// Adjoint scalars carried between reverse steps (FP64, device), and the
+// coefficients of the field update that the next kernel takes, in FP64 and
+// rounded once to FP32 (as every warp of it would form them).
+enum { kACl = 0, kACf, kACd, kAKp, kASg0, kASg1, kASv2, kASv3, kACoefs };
 struct AdjScalars {
     double ba, bad, bk0;     // adjoints of a, a' of the state being reached, and of kappa0
-    double cL, cF, cd, kp;   // forward coefficients of the step the next field update reverses
-    double bS[4];            // adjoint of that step's volume sums
+    double cd[kACoefs];      // cL/dx^2, cF, cdom, kappa of the step to reverse; -2 Sb0 /(dx^2 N^3), the same of Sb1, Sb2/N^3, Sb3/N^3
+    float cf[kACoefs];
     int status;
     unsigned int ticket;
+};
+template <typename T>
+__device__ __forceinline__ T adj_coef(const AdjScalars* as, int i);
+template <>
+__device__ __forceinline__ float adj_coef<float>(const AdjScalars* as, int i) { return as->cf[i]; }
+template <>
+__device__ __forceinline__ double adj_coef<double>(const AdjScalars* as, int i) { return as->cd[i]; }
+
+// The reverse of one step's scalar update is linear in the adjoints that come
+// into it, with coefficients that the forward pass fixes: those of every step
+// are formed by one launch before the sweep (a thread per step), so that the
+// serial end of a reverse step holds about 25 FP64 instructions (64 cycles each,
+// lat_common.cuh) where the whole chain of eq. scale in reverse held some 250
+// (128^3 FP32: 43.7 -> 32.9 us per reverse step, the field update's coefficients
+// rounded once instead of by every warp included).
+// With F, L, d, k the adjoints of cF, cL, cdom, kappa and Y that of y = a'_n +
+// a'_{n+1} from the a, a' update:
+//   Y' = Y + yF F,  c' = cF F + cY Y',  d' = d + V S2 c',  k' = k + V S3 c',
+//   a: aF F + aY Y' + aL L + aC c' + aD d' + aK k',  a': bY Y',  kappa0: pk k',
+//   Sb0 = Sb1 = s0 c',  Sb2 = V cdom c',  Sb3 = V kappa c'.
+struct AdjCoef {
+    double yF, cF, cY, V, S2, S3, aF, aY, aL, aC, aD, aK, bY, pk, s0;
+    double f_cL, f_cF, f_cd, f_kp;   // the forward coefficients of the step
 };
 
 template <typename T>
@@ -54,85 +81,52 @@ struct AdjBufs {
     T* pbo[2];        // adjoint of pi_k (out)
 };
 
-// Intermediate values of the forward scalar update of one step.
-struct ScaleFwd {
-    double c, q, alpha, y, ah, add, vpr, ea, eb;
-};
-
-// Recompute the forward scalar update from the scalars the step started from
-// (same formulas as scale_solve, with the intermediates kept). ia = 1/a.
-__device__ void scale_forward(const Model& M, const DevScalars& s, double ia, ScaleFwd& o)
-{
-    const double a = s.a;
-    o.vpr = s.cdom * s.S[2] + s.kappa * s.S[3];
-    o.ea = apow(a, ia, -2.0 * M.s - 2.0 * M.r - 1.0);
-    o.eb = apow(a, ia, 2.0 * M.s + 2.0);
-    o.c = M.g8A2 * o.ea * ((s.S[0] + s.S[1]) * (1.0 / 3.0) + o.eb * o.vpr);
-    o.q = -(M.s + 2.0) * ia;
-    o.alpha = M.dt * o.q * 0.25;
-    o.y = 2.0 * s.ad_half;
-    o.ah = s.ad_half;
-    o.add = s.add;
-}
-
-// Reverse of the scalar update of one step: given the adjoints of the
-// coefficients the kick used (bcL, bcF, bcd, bkp) and of y (from the a, a'
-// update), add to the adjoints of a, a' and kappa0 (ba, bad, bk0, kept in
-// registers by the caller) and produce those of S. One reciprocal of a and one
-// of the solve's denominator serve every quotient (the FP64 pipe is narrow and
-// this runs in one thread).
-__device__ void scale_reverse(const Model& M, const DevScalars& s, double bcL, double bcF, double bcd, double bkp,
-                              double by, double& ba_io, double& bad_io, double& bk0_io, double bS[4])
+// The reverse coefficients of the step that started from scalars s (eq. scale
+// and the coefficients of eq. scalar-evo: cF = r(s-r+2) h^2 + r a''/a with h =
+// a'_half / a, a'' = q a'_half^2 + c, a'_half = y / 2, y solving alpha y^2 - y +
+// gamma = 0 with gamma = 2a' + dt c, alpha = dt q / 4, q = -(s+2)/a,
+// c = K a^ec (T + a^ev V_pr), K = 8piG/A^2, T = (S0 + S1)/3).
+__device__ void adj_coefficients(const Model& M, const DevScalars& s, AdjCoef& o)
 {
     const double a = s.a, ia = 1.0 / a, ia2 = ia * ia;
-    double ba = 0.0, bad = 0.0;
-    for (int k = 0; k < 4; k++) bS[k] = 0.0;
+    o.yF = o.cF = o.cY = o.V = o.aF = o.aY = o.aL = o.aC = o.bY = o.s0 = 0.0;
+    o.S2 = s.S[2];
+    o.S3 = s.S[3];
     if (M.expansion) {
-        ScaleFwd o;
-        scale_forward(M, s, ia, o);
-        const double r = M.r, sx = M.s;
-        const double hh = o.ah * ia;
-        // cF = r(s-r+2) h^2 + r a''/a, h = a'_half / a
-        const double bh = bcF * 2.0 * r * (sx - r + 2.0) * hh;
-        const double badd = bcF * r * ia;
-        ba -= bcF * r * o.add * ia2;
-        double bah = bh * ia;
-        ba -= bh * o.ah * ia2;
-        // a'' = q a'_half^2 + c
-        double bq = badd * o.ah * o.ah;
-        bah += badd * 2.0 * o.q * o.ah;
-        double bc = badd;
-        // a'_half = y / 2; y solves alpha y^2 - y + gamma = 0 with gamma = 2a' + dt c
-        by += 0.5 * bah;
-        const double iden = 1.0 / (1.0 - 2.0 * o.alpha * o.y);
-        const double bgamma = by * iden, balpha = by * o.y * o.y * iden;
-        bq += balpha * M.dt * 0.25;
-        bad += 2.0 * bgamma;
-        bc += M.dt * bgamma;
-        ba += bq * (sx + 2.0) * ia2;
-        // cL = a^(-2s-2)
-        ba += bcL * (-2.0 * sx - 2.0) * apow(a, ia, -2.0 * sx - 3.0);
-        // c = K ea (T + eb vpr)
-        const double K = M.g8A2;
+        const double r = M.r, sx = M.s, dt = M.dt, ah = s.ad_half;
+        const double ec = -2.0 * sx - 2.0 * r - 1.0, ev = 2.0 * sx + 2.0;
+        const double vpr = s.cdom * s.S[2] + s.kappa * s.S[3];
+        const double ea = apow(a, ia, ec), eb = apow(a, ia, ev), K = M.g8A2;
         const double T = (s.S[0] + s.S[1]) * (1.0 / 3.0);
-        const double bea = bc * K * (T + o.eb * o.vpr);
-        const double bT = bc * K * o.ea;
-        const double beb = bc * K * o.ea * o.vpr;
-        const double bvpr = bc * K * o.ea * o.eb;
-        ba += bea * (-2.0 * sx - 2.0 * r - 1.0) * apow(a, ia, -2.0 * sx - 2.0 * r - 2.0);
-        ba += beb * (2.0 * sx + 2.0) * apow(a, ia, 2.0 * sx + 1.0);
-        bS[0] = bT * (1.0 / 3.0);
-        bS[1] = bT * (1.0 / 3.0);
-        bcd += bvpr * s.S[2];
-        bkp += bvpr * s.S[3];
-        bS[2] = bvpr * s.cdom;
-        bS[3] = bvpr * s.kappa;
+        const double q = -(sx + 2.0) * ia, y = 2.0 * ah, alpha = dt * q * 0.25;
+        const double c1 = 2.0 * r * (sx - r + 2.0) * (ah * ia);   // of h in cF
+        o.yF = 0.5 * (c1 * ia + 2.0 * q * ah * r * ia);
+        const double iden = 1.0 / (1.0 - 2.0 * alpha * y);
+        o.cF = r * ia;
+        o.cY = dt * iden;
+        o.bY = 2.0 * iden;
+        o.aF = (sx + 2.0) * ia2 * (r * ia * ah * ah) - r * s.add * ia2 - c1 * ah * ia2;
+        o.aY = (sx + 2.0) * ia2 * (y * y * iden * dt * 0.25);
+        o.aL = (-2.0 * sx - 2.0) * apow(a, ia, -2.0 * sx - 3.0);
+        o.aC = K * (T + eb * vpr) * ec * apow(a, ia, ec - 1.0) + K * ea * vpr * ev * apow(a, ia, ev - 1.0);
+        o.V = K * ea * eb;
+        o.s0 = K * ea * (1.0 / 3.0);
     }
-    // cdom = cdom0 a^pdom, kappa = kappa0 a^pint
-    ba += bcd * M.cdom0 * M.pdom * apow(a, ia, M.pdom - 1.0) + bkp * M.kappa0 * M.pint * apow(a, ia, M.pint - 1.0);
-    bk0_io += bkp * apow(a, ia, M.pint);
-    ba_io += ba;
-    bad_io += bad;
+    o.aD = M.cdom0 * M.pdom * apow(a, ia, M.pdom - 1.0);
+    o.aK = M.kappa0 * M.pint * apow(a, ia, M.pint - 1.0);
+    o.pk = apow(a, ia, M.pint);
+    o.f_cL = s.cL;
+    o.f_cF = s.cF;
+    o.f_cd = s.cdom;
+    o.f_kp = s.kappa;
+}
+__global__ void adj_coef_kernel(Model M, const DevScalars* hist, AdjCoef* coef, long long n)
+{
+    const long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (k >= n) return;
+    AdjCoef o;
+    adj_coefficients(M, hist[k], o);
+    coef[k] = o;
 }
 
 template <typename T>
@@ -143,104 +137,78 @@ __device__ __forceinline__ T powb1(T f, int beta)   // f^(beta-1), beta in {2, 4
 
 // Fold the per-thread sums of a reverse-step kernel (block reduction, then the
 // last block of the launch in fixed order) and run the FP64 scalar reverse of
-// step k-1 from them; hist = the scalars step k-1 started from. Writes the
-// coefficients and the adjoint of the sums that the next field update uses.
+// step k-1 from them; coef = that step's reverse coefficients. Writes the
+// coefficients that the next field update uses.
 template <typename T>
-__device__ void adj_finish(T acc[kSums], double* red, AdjScalars* as, const DevScalars* hist, double* partials,
+__device__ void adj_finish(T acc[kSums], double* red, AdjScalars* as, const AdjCoef* coef, double* partials,
                            const Model& M)
 {
-    double bs[kSums];
-    block_reduce(acc, red, bs);
-    __shared__ unsigned int is_last;
-    const int nblocks = gridDim.x * gridDim.y * gridDim.z;
-    const int bid = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z);
-    const int tid = threadIdx.x + blockDim.x * (threadIdx.y + blockDim.y * threadIdx.z);
-    if (tid == 0) {
-        for (int k = 0; k < kSums; k++) partials[(size_t)bid * kSums + k] = bs[k];
-        __threadfence();
-        is_last = atomicAdd(&as->ticket, 1u) == (unsigned int)nblocks - 1u;
-    }
-    __syncthreads();
-    if (!is_last) return;
-    __threadfence();
-    if (tid >= 32) return;
-    double v[kSums] = {0.0, 0.0, 0.0, 0.0};
-    // blocks tid, tid + 32, ... in order, four per pass so that their L2 loads
-    // are in flight together
-    const double2* p2 = reinterpret_cast<const double2*>(partials);   // kSums = 4 doubles per block
-    int b = tid;
-    for (; b + 96 < nblocks; b += 128) {
-        double2 x[4][2];
-#pragma unroll
-        for (int j = 0; j < 4; j++) {
-            x[j][0] = __ldcg(p2 + (size_t)(b + 32 * j) * 2);
-            x[j][1] = __ldcg(p2 + (size_t)(b + 32 * j) * 2 + 1);
+    __shared__ AdjCoef q;
+    __shared__ double base[4];   // ba, bk0, the incoming adjoint of y, bad without expansion
+    const int lane = linear_tid() & 31;
+    constexpr int kWords = (int)(sizeof(AdjCoef) / 8);
+    auto load = [&]() {
+        for (int i = lane; i < kWords; i += 32) reinterpret_cast<double*>(&q)[i] = reinterpret_cast<const double*>(coef)[i];
+        if (lane == 0) {
+            // reverse of a_{k} = a_{k-1} + dt a'_{k}, a'_{k} = y - a'_{k-1}
+            const double ba = as->ba, bad = as->bad;
+            base[0] = ba;
+            base[1] = as->bk0;
+            base[2] = M.expansion ? bad + M.dt * ba : 0.0;
+            base[3] = bad;
         }
-#pragma unroll
-        for (int j = 0; j < 4; j++) {
-            v[0] += x[j][0].x;
-            v[1] += x[j][0].y;
-            v[2] += x[j][1].x;
-            v[3] += x[j][1].y;
-        }
+    };
+    if (!block_ticket(acc, red, partials, &as->ticket, load, []() {})) return;
+    const double raw = last_block_fold(partials, red);
+    if (linear_tid() >= 32) return;
+    // the adjoints of cL, cF, cdom, kappa
+    const double in = raw * ((lane & 3) == 0 ? M.dt * M.inv_dx2 : (lane & 3) == 1 ? M.dt : -M.dt);
+    const double bL = __shfl_sync(0xffffffffu, in, 0), bF = __shfl_sync(0xffffffffu, in, 1);
+    const double bd = __shfl_sync(0xffffffffu, in, 2), bk = __shfl_sync(0xffffffffu, in, 3);
+    const double by = base[2] + q.yF * bF;
+    const double bc = q.cF * bF + q.cY * by;
+    const double bv = q.V * bc;
+    const double bd2 = bd + bv * q.S2, bk2 = bk + bv * q.S3;
+    const double ba = base[0] + (q.aF * bF + q.aY * by + q.aL * bL + q.aC * bc + q.aD * bd2 + q.aK * bk2);
+    const double bad = M.expansion ? q.bY * by - base[2] : base[3];
+    const double bk0 = base[1] + bk2 * q.pk;
+    // lanes 0..7: the coefficients of the next update
+    const double w = lane == kACl ? q.f_cL : lane == kACf ? q.f_cF : lane == kACd ? q.f_cd : lane == kAKp ? q.f_kp
+                     : lane == kASg0 || lane == kASg1 ? q.s0 * bc : bv * (lane == kASv2 ? q.f_cd : q.f_kp);
+    const double u = w * (lane == kACl ? M.inv_dx2 : lane == kASg0 || lane == kASg1 ? -2.0 * M.inv_dx2 : 1.0);
+    const double v = u * (lane >= kASg0 ? M.inv_sites : 1.0);
+    const bool finite = __all_sync(0xffffffffu, finite_bits(ba) && finite_bits(bad) && finite_bits(bk0) &&
+                                                    (lane >= kACoefs || finite_bits(v)));
+    if (lane < kACoefs) {
+        as->cd[lane] = v;
+        as->cf[lane] = (float)v;
     }
-    for (; b < nblocks; b += 32) {
-        const double2 x0 = __ldcg(p2 + (size_t)b * 2), x1 = __ldcg(p2 + (size_t)b * 2 + 1);
-        v[0] += x0.x;
-        v[1] += x0.y;
-        v[2] += x1.x;
-        v[3] += x1.y;
+    if (lane == 0) {
+        as->ticket = 0u;
+        as->ba = ba;
+        as->bad = bad;
+        as->bk0 = bk0;
+        if (!finite) as->status = LAT_ENONFINITE;
     }
-#pragma unroll
-    for (int k = 0; k < kSums; k++)
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_down_sync(0xffffffffu, v[k], o);
-    if (tid != 0) return;
-    // the scalar adjoints live in registers for the serial FP64 part
-    double ba = as->ba, bad = as->bad, bk0 = as->bk0;
-    as->ticket = 0u;
-    const DevScalars s = *hist;
-    // reverse of a_{k} = a_{k-1} + dt a'_{k}, a'_{k} = y - a'_{k-1}
-    double by = 0.0;
-    if (M.expansion) {
-        by = bad + M.dt * ba;
-        bad = -by;
-    }
-    const double bcL = M.dt * v[0] * M.inv_dx2, bcF = M.dt * v[1], bcd = -M.dt * v[2], bkp = -M.dt * v[3];
-    double bS[4];
-    scale_reverse(M, s, bcL, bcF, bcd, bkp, by, ba, bad, bk0, bS);
-    bool finite = isfinite(ba) && isfinite(bad) && isfinite(bk0);
-    for (int k = 0; k < 4; k++) {
-        as->bS[k] = bS[k];
-        finite = finite && isfinite(bS[k]);
-    }
-    as->ba = ba;
-    as->bad = bad;
-    as->bk0 = bk0;
-    as->cL = s.cL;
-    as->cF = s.cF;
-    as->cd = s.cdom;
-    as->kp = s.kappa;
-    if (!finite) as->status = LAT_ENONFINITE;
-    __threadfence();
 }
 
 // Reverse step kernel, one site per thread (any N). UPDATE: reverse the field update of step k (outputs fbo,
 // pbo); always: if fm is given, the four sums of step k-1 from pt' = pb_k + dt fb_k
 // (without UPDATE, pb + dt fb of the inputs), folded by the last block into the
-// scalar reverse of step k-1 (hist = the scalars step k-1 started from).
+// scalar reverse of step k-1 (coef = that step's reverse coefficients).
 template <typename T, bool UPDATE>
 __global__ void __launch_bounds__(kAdjThreads) adj_step_kernel(AdjBufs<T> B, Model M, AdjScalars* as,
-                                                               const DevScalars* hist, double* partials)
+                                                               const AdjCoef* coef, double* partials)
 {
     __shared__ double red[32 * kSums];
+    chain_begin();
     if (as->status != LAT_OK) return;
     const int n = M.n;
     const long long nn = (long long)n * n, n3 = nn * n;
     const T dt = (T)M.dt;
-    const T cLs = (T)(as->cL * M.inv_dx2), cF = (T)as->cF, cd = (T)as->cd, kp = (T)as->kp;
-    const T sg0 = (T)(-2.0 * as->bS[0] * M.inv_dx2 * M.inv_sites), sg1 = (T)(-2.0 * as->bS[1] * M.inv_dx2 * M.inv_sites);
-    const T sv2 = (T)(as->bS[2] * M.inv_sites), sv3 = (T)(as->bS[3] * M.inv_sites);
+    const T cLs = adj_coef<T>(as, kACl), cF = adj_coef<T>(as, kACf), cd = adj_coef<T>(as, kACd), kp = adj_coef<T>(as, kAKp);
+    const T sg0 = adj_coef<T>(as, kASg0), sg1 = adj_coef<T>(as, kASg1);
+    const T sv2 = adj_coef<T>(as, kASv2), sv3 = adj_coef<T>(as, kASv3);
     const int beta = M.beta;
     const bool sums = B.fm[0] != nullptr;
     T acc[kSums] = {T(0), T(0), T(0), T(0)};
@@ -306,7 +274,7 @@ __global__ void __launch_bounds__(kAdjThreads) adj_step_kernel(AdjBufs<T> B, Mod
         }
     }
     if (!sums) return;
-    adj_finish(acc, red, as, hist, partials, M);
+    adj_finish(acc, red, as, coef, partials, M);
 }
 
 // Reverse step kernel as a z-march (N a multiple of 32): a 32 x 8 tile of
@@ -329,13 +297,14 @@ constexpr size_t adj_march_smem()
 
 template <typename T>
 __global__ void __launch_bounds__(kMX * kMY, sizeof(T) == 4 ? 3 : 2)
-    adj_march_kernel(AdjBufs<T> B, Model M, AdjScalars* as, const DevScalars* hist, double* partials, int nzc)
+    adj_march_kernel(AdjBufs<T> B, Model M, AdjScalars* as, const AdjCoef* coef, double* partials, int nzc)
 {
     __shared__ double red[32 * kSums];
     extern __shared__ __align__(16) unsigned char smem_raw[];
     T (*stage)[8][kMX * kMY] = reinterpret_cast<T (*)[8][kMX * kMY]>(smem_raw);
     T (*tiles)[6][kMY + 2][kMX + 2] =
         reinterpret_cast<T (*)[6][kMY + 2][kMX + 2]>(smem_raw + sizeof(T) * kStage * 8 * kMX * kMY);
+    chain_begin();
     if (as->status != LAT_OK) return;
     const int n = M.n;
     const uint32_t nn = (uint32_t)n * n;
@@ -344,9 +313,9 @@ __global__ void __launch_bounds__(kMX * kMY, sizeof(T) == 4 ? 3 : 2)
     const int z0 = (int)((long long)blockIdx.z * n / nzc);
     const int nz = (int)((long long)(blockIdx.z + 1) * n / nzc) - z0;
     const T dt = (T)M.dt;
-    const T cLs = (T)(as->cL * M.inv_dx2), cF = (T)as->cF, cd = (T)as->cd, kp = (T)as->kp;
-    const T sg0 = (T)(-2.0 * as->bS[0] * M.inv_dx2 * M.inv_sites), sg1 = (T)(-2.0 * as->bS[1] * M.inv_dx2 * M.inv_sites);
-    const T sv2 = (T)(as->bS[2] * M.inv_sites), sv3 = (T)(as->bS[3] * M.inv_sites);
+    const T cLs = adj_coef<T>(as, kACl), cF = adj_coef<T>(as, kACf), cd = adj_coef<T>(as, kACd), kp = adj_coef<T>(as, kAKp);
+    const T sg0 = adj_coef<T>(as, kASg0), sg1 = adj_coef<T>(as, kASg1);
+    const T sv2 = adj_coef<T>(as, kASv2), sv3 = adj_coef<T>(as, kASv3);
     const int beta = M.beta;
     const bool sums = B.fm[0] != nullptr;
     // raw arrays: 0,1 pb; 2,3 fb; 4,5 f_k; 6,7 f_{k-1}
@@ -474,7 +443,7 @@ __global__ void __launch_bounds__(kMX * kMY, sizeof(T) == 4 ? 3 : 2)
     }
     cp_async_wait(0);
     if (!sums) return;
-    adj_finish(acc, red, as, hist, partials, M);
+    adj_finish(acc, red, as, coef, partials, M);
 }
 
 // FP32 reverse step with two x sites per thread (N a multiple of 64): the
@@ -495,11 +464,12 @@ struct AdjPairSmem {
 };
 
 __global__ void __launch_bounds__(kPX * kPY, 2)
-    adj_pair_kernel(AdjBufs<float> B, Model M, AdjScalars* as, const DevScalars* hist, double* partials, int nzc)
+    adj_pair_kernel(AdjBufs<float> B, Model M, AdjScalars* as, const AdjCoef* coef, double* partials, int nzc)
 {
     __shared__ double red[32 * kSums];
     extern __shared__ __align__(16) unsigned char smem_raw[];
     AdjPairSmem& SM = *reinterpret_cast<AdjPairSmem*>(smem_raw);
+    chain_begin();
     if (as->status != LAT_OK) return;
     const int n = M.n;
     const uint32_t nn = (uint32_t)n * n;
@@ -509,13 +479,9 @@ __global__ void __launch_bounds__(kPX * kPY, 2)
     const int nz = (int)((long long)(blockIdx.z + 1) * n / nzc) - z0;
     const float dts = (float)M.dt;
     const F2 dt = mk2(dts, dts);
-    const float cLv = (float)(as->cL * M.inv_dx2);
-    const F2 cLs = mk2(cLv, cLv), cF = mk2((float)as->cF, (float)as->cF);
-    const F2 cd = mk2((float)as->cd, (float)as->cd), kp = mk2((float)as->kp, (float)as->kp);
-    const float g0v = (float)(-2.0 * as->bS[0] * M.inv_dx2 * M.inv_sites), g1v = (float)(-2.0 * as->bS[1] * M.inv_dx2 * M.inv_sites);
-    const F2 sg0 = mk2(g0v, g0v), sg1 = mk2(g1v, g1v);
-    const F2 sv2 = mk2((float)(as->bS[2] * M.inv_sites), (float)(as->bS[2] * M.inv_sites));
-    const F2 sv3 = mk2((float)(as->bS[3] * M.inv_sites), (float)(as->bS[3] * M.inv_sites));
+    auto both = [&](int i) { return mk2(as->cf[i], as->cf[i]); };
+    const F2 cLs = both(kACl), cF = both(kACf), cd = both(kACd), kp = both(kAKp);
+    const F2 sg0 = both(kASg0), sg1 = both(kASg1), sv2 = both(kASv2), sv3 = both(kASv3);
     const F2 two = mk2(2.0f, 2.0f), three = mk2(3.0f, 3.0f);
     const bool quartic = M.beta == 4;
     const bool sums = B.fm[0] != nullptr;
@@ -688,7 +654,7 @@ __global__ void __launch_bounds__(kPX * kPY, 2)
     if (!sums) return;
     float v[kSums] = {lo2(acc[0]) + hi2(acc[0]), lo2(acc[1]) + hi2(acc[1]), lo2(acc[2]) + hi2(acc[2]),
                       lo2(acc[3]) + hi2(acc[3])};
-    adj_finish(v, red, as, hist, partials, M);
+    adj_finish(v, red, as, coef, partials, M);
 }
 
 // J = <f1^2> (volume mean of chi squared) per block, and its gradient 2 f1 / N^3.
@@ -885,20 +851,28 @@ struct LogGuard {
     }
 };
 
-// Device allocations of one reverse-mode call, freed together.
+// The device memory of one reverse-mode call: one allocation, the arrays cut from
+// it in order (ten allocations and frees of a 128^3 call of 100 steps: 1.09 ms,
+// one: 0.38).
 struct Scratch {
-    std::vector<void*> ptrs;
-    ~Scratch()
-    {
-        for (void* p : ptrs) cudaFree(p);
-    }
+    void* base = nullptr;
+    std::vector<std::pair<void**, size_t>> parts;
+    ~Scratch() { cudaFree(base); }
     template <typename P>
-    bool alloc(P** out, size_t bytes)
+    void want(P** out, size_t bytes)
     {
-        void* p = nullptr;
-        if (cudaMalloc(&p, std::max<size_t>(bytes, 16)) != cudaSuccess) return false;
-        ptrs.push_back(p);
-        *out = static_cast<P*>(p);
+        parts.emplace_back((void**)out, (std::max<size_t>(bytes, 16) + 255) / 256 * 256);
+    }
+    bool alloc()
+    {
+        size_t total = 0;
+        for (auto& p : parts) total += p.second;
+        if (cudaMalloc(&base, total) != cudaSuccess) return false;
+        char* at = (char*)base;
+        for (auto& p : parts) {
+            *p.first = at;
+            at += p.second;
+        }
         return true;
     }
 };
@@ -948,13 +922,19 @@ lat_status vjp_impl(lat_handle* h, int64_t n, int64_t ckpt_every, T* fb_user, T*
     T *ck = nullptr, *seg = nullptr, *adj1 = nullptr, *fin = nullptr;
     DevScalars *ck_sc = nullptr, *hist = nullptr, *fin_sc = nullptr;
     AdjScalars* as = nullptr;
+    AdjCoef* coef = nullptr;
     double* part = nullptr;
-    if (!S.alloc(&ck, (size_t)nck * 6 * ab) || !S.alloc(&ck_sc, (size_t)nck * sizeof(DevScalars)) ||
-        !S.alloc(&hist, (size_t)(n + 1) * sizeof(DevScalars)) || !S.alloc(&seg, (size_t)K * 2 * ab) ||
-        !S.alloc(&adj1, 4 * ab) || !S.alloc(&fin, 4 * ab) || !S.alloc(&fin_sc, sizeof(DevScalars)) ||
-        !S.alloc(&as, sizeof(AdjScalars)) ||
-        !S.alloc(&part, std::max(nparts * kSums, (size_t)nb * kFracSums) * sizeof(double)))
-        return LAT_ENOMEM;
+    S.want(&ck, (size_t)nck * 6 * ab);
+    S.want(&ck_sc, (size_t)nck * sizeof(DevScalars));
+    S.want(&hist, (size_t)(n + 1) * sizeof(DevScalars));
+    S.want(&seg, (size_t)(K + 1) * 2 * ab);
+    S.want(&adj1, 4 * ab);
+    S.want(&fin, 4 * ab);
+    S.want(&fin_sc, sizeof(DevScalars));
+    S.want(&as, sizeof(AdjScalars));
+    S.want(&coef, (size_t)std::max<int64_t>(n, 1) * sizeof(AdjCoef));
+    S.want(&part, std::max(nparts * kSums, (size_t)nb * kFracSums) * sizeof(double));
+    if (!S.alloc()) return LAT_ENOMEM;
     Bufs<T> hb = bufs_of<T>(h);
     auto arr = [&](T* base, size_t i) { return base + i * N3; };
 
@@ -970,6 +950,19 @@ lat_status vjp_impl(lat_handle* h, int64_t n, int64_t ckpt_every, T* fb_user, T*
         guard.armed = true;
     }
     LAT_CUDA(cudaMemcpyAsync(hist, h->sc, sizeof(DevScalars), cudaMemcpyDeviceToDevice, st));
+    // The fields of the last segment are kept where its reversal reads them (pair
+    // k - c of seg holds f_k, as in a recomputation), so it is not recomputed.
+    const int64_t clast = n > 0 ? (nck - 1) * K : 0;
+    // buffers of step k of a segment that starts at step c: the fields in seg
+    auto seg_bufs = [&](int64_t k, int64_t c) {
+        Bufs<T> b = hb;
+        const int par = (int)((s0.step + k) & 1);
+        for (int f = 0; f < 2; f++) {
+            b.f[par][f] = arr(seg, (size_t)(k - c) * 2 + f);
+            b.f[1 - par][f] = arr(seg, (size_t)(k - c + 1) * 2 + f);
+        }
+        return b;
+    };
     for (int64_t k = 0; k < n; k++) {
         const int par = (int)((s0.step + k) & 1);
         if (k % K == 0) {
@@ -980,11 +973,17 @@ lat_status vjp_impl(lat_handle* h, int64_t n, int64_t ckpt_every, T* fb_user, T*
                 if (k > 0) LAT_CUDA(cudaMemcpyAsync(c + (4 + f) * N3, hb.f[1 - par][f], ab, cudaMemcpyDeviceToDevice, st));
             }
             LAT_CUDA(cudaMemcpyAsync(ck_sc + k / K, h->sc, sizeof(DevScalars), cudaMemcpyDeviceToDevice, st));
+            if (k == clast)
+                for (int f = 0; f < 2; f++)
+                    LAT_CUDA(cudaMemcpyAsync(arr(seg, f), hb.f[par][f], ab, cudaMemcpyDeviceToDevice, st));
         }
-        LAT_CUDA(launch_step_with<T>(h, hb, k % K != 0));
+        LAT_CUDA(launch_step_with<T>(h, k < clast ? hb : seg_bufs(k, clast), k % K != 0));
     }
     LAT_TRY(guard.clear());
     const int parN = (int)((s0.step + n) & 1);
+    if (n > 0)   // f_n back into the handle's own set
+        for (int f = 0; f < 2; f++)
+            LAT_CUDA(cudaMemcpyAsync(hb.f[parN][f], arr(seg, (size_t)(n - clast) * 2 + f), ab, cudaMemcpyDeviceToDevice, st));
     for (int f = 0; f < 2; f++) {
         LAT_CUDA(cudaMemcpyAsync(fin + f * N3, hb.f[parN][f], ab, cudaMemcpyDeviceToDevice, st));
         LAT_CUDA(cudaMemcpyAsync(fin + (2 + f) * N3, hb.p[parN][f], ab, cudaMemcpyDeviceToDevice, st));
@@ -1067,55 +1066,49 @@ lat_status vjp_impl(lat_handle* h, int64_t n, int64_t ckpt_every, T* fb_user, T*
         return b;
     };
     if (n > 0) {
-        // sums of the last step from the final adjoint and f_{n-1}, still in
-        // the other ping-pong buffer
-        T* fm_last = seg;   // f_{n-1} copied next to the segment storage
-        for (int f = 0; f < 2; f++)
-            LAT_CUDA(cudaMemcpyAsync(fm_last + f * N3, hb.f[1 - parN][f], ab, cudaMemcpyDeviceToDevice, st));
-        adj_step_kernel<T, false><<<nb, kAdjThreads, 0, st>>>(adj_bufs(nullptr, fm_last), M, as, hist + (n - 1), part);
+        adj_coef_kernel<<<(unsigned)((n + 31) / 32), 32, 0, st>>>(M, hist, coef, n);
+        LAT_CUDA(cudaGetLastError());
+        // sums of the last step from the final adjoint and f_{n-1}
+        const T* fm_last = arr(seg, (size_t)(n - 1 - clast) * 2);
+        adj_step_kernel<T, false><<<nb, kAdjThreads, 0, st>>>(adj_bufs(nullptr, fm_last), M, as, coef + (n - 1), part);
         LAT_CUDA(cudaGetLastError());
     }
     for (int64_t sgi = nck - 1; sgi >= 0; sgi--) {
         const int64_t c = sgi * K, e = std::min<int64_t>(c + K, n);
         const T* cp = arr(ck, (size_t)sgi * 6);
-        // restore the checkpoint and recompute f_c .. f_{e-1} into the segment storage
-        const int parc = (int)((s0.step + c) & 1);
-        for (int f = 0; f < 2; f++) {
-            LAT_CUDA(cudaMemcpyAsync(seg + f * N3, cp + f * N3, ab, cudaMemcpyDeviceToDevice, st));
-            LAT_CUDA(cudaMemcpyAsync(hb.p[parc][f], cp + (2 + f) * N3, ab, cudaMemcpyDeviceToDevice, st));
-        }
-        LAT_CUDA(cudaMemcpyAsync(h->sc, ck_sc + sgi, sizeof(DevScalars), cudaMemcpyDeviceToDevice, st));
-        guard.armed = true;   // the checkpoint's block carries the history pointer
-        LAT_TRY(guard.clear());
-        for (int64_t k = c; k + 1 < e; k++) {
-            const int par = (int)((s0.step + k) & 1);
-            Bufs<T> b = hb;
+        if (c != clast) {
+            // restore the checkpoint and recompute f_c .. f_{e-1} into the segment storage
+            const int parc = (int)((s0.step + c) & 1);
             for (int f = 0; f < 2; f++) {
-                b.f[par][f] = arr(seg, (size_t)(k - c) * 2 + f);
-                b.f[1 - par][f] = arr(seg, (size_t)(k - c + 1) * 2 + f);
+                LAT_CUDA(cudaMemcpyAsync(seg + f * N3, cp + f * N3, ab, cudaMemcpyDeviceToDevice, st));
+                LAT_CUDA(cudaMemcpyAsync(hb.p[parc][f], cp + (2 + f) * N3, ab, cudaMemcpyDeviceToDevice, st));
             }
-            LAT_CUDA(launch_step_with<T>(h, b, k > c));
+            LAT_CUDA(cudaMemcpyAsync(h->sc, ck_sc + sgi, sizeof(DevScalars), cudaMemcpyDeviceToDevice, st));
+            guard.armed = true;   // the checkpoint's block carries the history pointer
+            LAT_TRY(guard.clear());
+            for (int64_t k = c; k + 1 < e; k++) LAT_CUDA(launch_step_with<T>(h, seg_bufs(k, c), k > c));
         }
         // reverse steps e-1 .. c
         for (int64_t k = e - 1; k >= c; k--) {
             const T* fk = arr(seg, (size_t)(k - c) * 2);
             const T* fm = k > c ? arr(seg, (size_t)(k - c - 1) * 2) : (k > 0 ? cp + 4 * N3 : nullptr);
+            AdjBufs<T> ab2 = adj_bufs(fk, fm);
+            const AdjCoef* q = k > 0 ? coef + (k - 1) : coef;
+            int chunks = nzc;
+            Model Mv = M;
+            void* args[] = {(void*)&ab2, (void*)&Mv, (void*)&as, (void*)&q, (void*)&part, (void*)&chunks};
+            const bool chain = k < e - 1;   // behind the reverse step of k + 1
             if constexpr (sizeof(T) == 4) {
-                if (pair) {
-                    adj_pair_kernel<<<mgrid, dim3(kPX, kPY), sizeof(AdjPairSmem), st>>>(
-                        adj_bufs(fk, fm), M, as, k > 0 ? hist + (k - 1) : hist, part, nzc);
-                    LAT_CUDA(cudaGetLastError());
-                    cur = 1 - cur;
-                    continue;
-                }
+                if (pair)
+                    LAT_CUDA(launch_chained((const void*)adj_pair_kernel, mgrid, dim3(kPX, kPY), args, sizeof(AdjPairSmem),
+                                            st, chain));
             }
             if (march)
-                adj_march_kernel<T><<<mgrid, dim3(kMX, kMY), adj_march_smem<T>(), st>>>(
-                    adj_bufs(fk, fm), M, as, k > 0 ? hist + (k - 1) : hist, part, nzc);
-            else
-                adj_step_kernel<T, true><<<nb, kAdjThreads, 0, st>>>(adj_bufs(fk, fm), M, as,
-                                                                     k > 0 ? hist + (k - 1) : hist, part);
-            LAT_CUDA(cudaGetLastError());
+                LAT_CUDA(launch_chained((const void*)adj_march_kernel<T>, mgrid, dim3(kMX, kMY), args, adj_march_smem<T>(),
+                                        st, chain));
+            else if (!pair)
+                LAT_CUDA(launch_chained((const void*)adj_step_kernel<T, true>, dim3(nb), dim3(kAdjThreads), args, 0, st,
+                                        chain));
             cur = 1 - cur;
         }
     }
