@@ -125,18 +125,15 @@ cudaError_t launch_step27w(const Bufs<T>& b, const Model& M, DevScalars* sc, dou
                            cudaStream_t st);
 
 // Initial conditions (off the timed path).
-struct InitWork {
-    double* re;      // N^3 doubles
-    double* keep;    // N^3 doubles
-    void* spec;      // N*N*(N/2+1) complex doubles
-    int fft_fwd, fft_inv;  // cufft handles
-};
 template <typename T>
 cudaError_t launch_init_combine(const Bufs<T>& b, int field, const double* df, const double* dp, double fh,
                                 double ph, double r_h0, double half_dt, int n, cudaStream_t st);
+// the noise and axis tables of one side, init_tables_bytes(n) bytes on the device
+size_t init_tables_bytes(int n);
+cudaError_t launch_init_tables(void* tables, int n, cudaStream_t st);
 cudaError_t launch_white_noise(double* out, int n, uint64_t seed, uint32_t field, uint32_t quantity,
-                               cudaStream_t st);
-cudaError_t launch_spectral_scale(void* spec, int n, double dx, double meff2, double amp, double kcut,
+                               const void* tables, cudaStream_t st);
+cudaError_t launch_spectral_scale(void* spec, int n, const void* tables, double dx, double meff2, double amp, double kcut,
                                   int quantity, int stencil, cudaStream_t st);
 
 // Split storage (lat_split.cu): a[i] += delta (in FP64, rounded once), and
