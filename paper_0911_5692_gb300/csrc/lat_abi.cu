@@ -361,7 +361,7 @@ lat_status create_common(const lat_params* params, void* stream, void* const buf
     if (st == LAT_OK && cudaMalloc((void**)&h->sc, sizeof(DevScalars)) != cudaSuccess) st = LAT_ENOMEM;
     if (st == LAT_OK && cudaMalloc((void**)&h->partials, h->partials_cap * sizeof(double)) != cudaSuccess)
         st = LAT_ENOMEM;
-    if (st == LAT_OK && cudaMalloc((void**)&h->means, 2 * sizeof(double)) != cudaSuccess) st = LAT_ENOMEM;
+    if (st == LAT_OK && cudaMalloc((void**)&h->means, (kEnergySums + 2) * sizeof(double)) != cudaSuccess) st = LAT_ENOMEM;
     if (st == LAT_OK) {
         DevScalars s;
         std::memset(&s, 0, sizeof(s));
@@ -432,6 +432,7 @@ void lat_destroy(lat_handle* h)
     if (h->sc) cudaFree(h->sc);
     if (h->partials) cudaFree(h->partials);
     if (h->means) cudaFree(h->means);
+    if (h->have_fft) cufftDestroy(h->fft);
     for (cudaEvent_t e : h->host_down_ev)
         if (e) cudaEventDestroy(e);
     if (h->host_up_done) cudaEventDestroy(h->host_up_done);
@@ -1037,29 +1038,15 @@ lat_status lat_energies(lat_handle* h, lat_energy_report* out)
     if (h->slab) return LAT_ESTATE;
     LAT_TRY(ensure_prepared(h));
     const Model& M = h->M;
-    const int nb = energies_grid_blocks(M.n);
-    std::vector<double> part((size_t)nb * kEnergySums);
-    double tot[kEnergySums];
-    for (int pass = 0; pass < 2; pass++) {
-        cudaError_t e = h->prec == 32 ? launch_energies<float>(bufs_of<float>(h), M, h->sc, h->partials, h->means, pass, h->stream)
-                                      : launch_energies<double>(bufs_of<double>(h), M, h->sc, h->partials, h->means, pass, h->stream);
-        LAT_CUDA(e);
-        LAT_CUDA(cudaMemcpyAsync(part.data(), h->partials, part.size() * sizeof(double), cudaMemcpyDeviceToHost,
-                                 h->stream));
-        LAT_CUDA(cudaStreamSynchronize(h->stream));
-        double acc[kEnergySums] = {0, 0, 0, 0, 0, 0, 0};
-        for (int b = 0; b < nb; b++)
-            for (int k = 0; k < kEnergySums; k++) acc[k] += part[(size_t)b * kEnergySums + k];
-        if (pass == 0) {
-            for (int k = 0; k < kEnergySums; k++) tot[k] = acc[k] * M.inv_sites;
-            LAT_CUDA(cudaMemcpyAsync(h->means, &tot[5], 2 * sizeof(double), cudaMemcpyHostToDevice, h->stream));
-        } else {
-            out->var[0] = acc[5] * M.inv_sites;
-            out->var[1] = acc[6] * M.inv_sites;
-        }
-    }
+    cudaError_t e = h->prec == 32 ? launch_energies<float>(bufs_of<float>(h), M, h->sc, h->partials, h->means, h->stream)
+                                  : launch_energies<double>(bufs_of<double>(h), M, h->sc, h->partials, h->means, h->stream);
+    LAT_CUDA(e);
+    double tot[kEnergySums + 2];
+    LAT_CUDA(cudaMemcpyAsync(tot, h->means, sizeof(tot), cudaMemcpyDeviceToHost, h->stream));
     DevScalars s;
     LAT_TRY(read_scalars(h, &s));
+    out->var[0] = tot[kEnergySums];
+    out->var[1] = tot[kEnergySums + 1];
     const double a = s.a;
     const double hh = M.expansion ? s.ad_half / a : 0.0;
     const double cg = std::pow(a, -2.0 * M.s - 2.0);
@@ -1105,52 +1092,56 @@ lat_status lat_spectrum(lat_handle* h, int field, int nbins, double* k_out, doub
     LAT_TRY(read_scalars(h, &s));
     const int par = (int)(s.step & 1);
     const size_t nspec = (size_t)n * n * (n / 2 + 1);
-    const int nb = spectrum_grid_blocks(n);
-    double* re = nullptr;
-    void* spec = nullptr;
-    double* part = nullptr;
+    // one allocation: the field in FP64, its spectrum, the shells' scratch and sums
+    auto up = [](size_t bytes) { return (bytes + 255) / 256 * 256; };
+    const size_t b_re = up(h->nsites * sizeof(double)), b_spec = up(nspec * sizeof(cufftDoubleComplex));
+    const size_t b_part = up(spectrum_scratch(n, nbins) * sizeof(double));
+    char* arena = nullptr;
     lat_status st = LAT_OK;
-    cufftHandle fwd = 0;
-    bool have = false;
-    if (cudaMalloc((void**)&re, h->nsites * sizeof(double)) != cudaSuccess ||
-        cudaMalloc(&spec, nspec * sizeof(cufftDoubleComplex)) != cudaSuccess ||
-        cudaMalloc((void**)&part, (size_t)nb * 3 * nbins * sizeof(double)) != cudaSuccess)
-        st = LAT_ENOMEM;
-    if (st == LAT_OK) {
+    if (!h->have_fft) {
+        cufftHandle plan = 0;
+        if (cufftCreate(&plan) != CUFFT_SUCCESS) return LAT_ECUDA;
+        if (cufftSetAutoAllocation(plan, 0) != CUFFT_SUCCESS ||
+            cufftMakePlan3d(plan, n, n, n, CUFFT_D2Z, &h->fft_work) != CUFFT_SUCCESS) {
+            cufftDestroy(plan);
+            return LAT_ECUDA;
+        }
+        h->fft = plan;
+        h->have_fft = true;
+    }
+    const size_t b_sums = up((size_t)3 * nbins * sizeof(double));
+    if (cudaMalloc((void**)&arena, b_re + b_spec + b_part + b_sums + h->fft_work) != cudaSuccess) return LAT_ENOMEM;
+    double* re = (double*)arena;
+    void* spec = arena + b_re;
+    double *part = (double*)(arena + b_re + b_spec), *sums = (double*)(arena + b_re + b_spec + b_part);
+    {
         const void* src = h->buf[4 * par + field];
-        cudaError_t e = h->prec == 32 ? launch_to_double<float>((const float*)src, re, h->nsites, h->stream)
-                                      : launch_to_double<double>((const double*)src, re, h->nsites, h->stream);
-        if (e == cudaSuccess) e = launch_shift<double>(re, h->nsites, whole_offset(h, s, field, 0), h->stream);
+        const double off = whole_offset(h, s, field, 0);
+        cudaError_t e = h->prec == 32 ? launch_to_double<float>((const float*)src, re, h->nsites, off, h->stream)
+                                      : launch_to_double<double>((const double*)src, re, h->nsites, off, h->stream);
         if (e != cudaSuccess) st = LAT_ECUDA;
     }
-    if (st == LAT_OK) {
-        if (cufftPlan3d(&fwd, n, n, n, CUFFT_D2Z) != CUFFT_SUCCESS) st = LAT_ECUDA;
-        else have = true;
-    }
-    if (st == LAT_OK && cufftSetStream(fwd, h->stream) != CUFFT_SUCCESS) st = LAT_ECUDA;
-    if (st == LAT_OK && cufftExecD2Z(fwd, re, (cufftDoubleComplex*)spec) != CUFFT_SUCCESS) st = LAT_ECUDA;
-    if (st == LAT_OK && launch_spectrum_bins(spec, n, h->p.L, nbins, part, h->stream) != cudaSuccess) st = LAT_ECUDA;
+    if (st == LAT_OK && (cufftSetStream(h->fft, h->stream) != CUFFT_SUCCESS ||
+                         (h->fft_work && cufftSetWorkArea(h->fft, arena + b_re + b_spec + b_part + b_sums) != CUFFT_SUCCESS) ||
+                         cufftExecD2Z(h->fft, re, (cufftDoubleComplex*)spec) != CUFFT_SUCCESS))
+        st = LAT_ECUDA;
+    if (st == LAT_OK && launch_spectrum_bins(spec, n, h->p.L, nbins, part, sums, h->stream) != cudaSuccess) st = LAT_ECUDA;
     std::vector<double> hp;
     if (st == LAT_OK) {
-        hp.resize((size_t)nb * 3 * nbins);
-        if (cudaMemcpyAsync(hp.data(), part, hp.size() * sizeof(double), cudaMemcpyDeviceToHost, h->stream) != cudaSuccess ||
+        hp.resize((size_t)3 * nbins);
+        if (cudaMemcpyAsync(hp.data(), sums, hp.size() * sizeof(double), cudaMemcpyDeviceToHost, h->stream) != cudaSuccess ||
             cudaStreamSynchronize(h->stream) != cudaSuccess)
             st = LAT_ECUDA;
     }
     if (st == LAT_OK) {
         for (int b = 0; b < nbins; b++) {
-            double pp = 0.0, kk = 0.0, cc = 0.0;
-            for (int blk = 0; blk < nb; blk++) {
-                const double* row = hp.data() + (size_t)blk * 3 * nbins;
-                pp += row[b]; kk += row[nbins + b]; cc += row[2 * nbins + b];
-            }
+            const double pp = hp[b], kk = hp[nbins + b], cc = hp[2 * nbins + b];
             count_out[b] = (int64_t)std::llround(cc);
             p_out[b] = cc > 0.0 ? pp / cc : 0.0;
             k_out[b] = cc > 0.0 ? kk / cc : 0.0;
         }
     }
-    if (have) cufftDestroy(fwd);
-    cudaFree(re); cudaFree(spec); cudaFree(part);
+    cudaFree(arena);
     if (st != LAT_OK) return st;
     return (lat_status)s.status;
 }

@@ -17,13 +17,19 @@ struct lat_handle {
     lat::DevScalars* sc;      // device
     double* partials;    // device, per-block sums
     size_t partials_cap; // doubles
-    double* means;       // device, 2 doubles
+    double* means;       // device, kEnergySums + 2 doubles: the averages of lat_energies
     bool dirty;          // sums and coefficients must be recomputed
     int variant;         // 2 = plane-ring z-march over full rows, 4 = over x tiles
     int ty, zr;
     lat::MarchConfig mcfg;
     cudaGraphExec_t graph;
     int graph_steps;
+    // lat_spectrum's transform, kept from its first call to lat_destroy (no device
+    // memory: its work area comes from each call's own; a plan costs 0.55 ms of a
+    // 256^3 call's 2.9)
+    int fft;             // cufftHandle
+    bool have_fft;
+    size_t fft_work;     // bytes
     bool slab;           // a z-slab of a larger lattice (lat_slab_create)
     int slab_z0, slab_nzl;
     // lat_evolve_host: one copy stream per direction, its events and the

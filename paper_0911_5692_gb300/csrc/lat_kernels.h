@@ -148,11 +148,13 @@ cudaError_t launch_sum2(const T* a, const T* b, size_t count, double* partials, 
 // Diagnostics (off the timed path).
 constexpr int kEnergySums = 7;
 int energies_grid_blocks(int n);
+// out (device, kEnergySums + 2 doubles): the averages of the energy sums, the
+// fields' means last, then the variances about them
 template <typename T>
-cudaError_t launch_energies(const Bufs<T>& b, const Model& M, const DevScalars* sc, double* partials,
-                            const double* means, int pass, cudaStream_t st);
+cudaError_t launch_energies(const Bufs<T>& b, const Model& M, const DevScalars* sc, double* partials, double* out,
+                            cudaStream_t st);
 template <typename T>
-cudaError_t launch_to_double(const T* src, double* dst, size_t count, cudaStream_t st);
+cudaError_t launch_to_double(const T* src, double* dst, size_t count, double offset, cudaStream_t st);
 // energy density and pressure at every site (eq. rho-pres per site)
 template <typename T>
 cudaError_t launch_energy_field(const Bufs<T>& b, const Model& M, const DevScalars* sc, T* rho, T* pres,
@@ -162,8 +164,10 @@ cudaError_t launch_energy_field(const Bufs<T>& b, const Model& M, const DevScala
 // whose last block solves the next step's coefficients (lat_lform.cu).
 template <typename T>
 cudaError_t launch_lform(const Bufs<T>& b, const Model& M, DevScalars* sc, double* partials, cudaStream_t st);
-int spectrum_grid_blocks(int n);
-cudaError_t launch_spectrum_bins(const void* spec, int n, double L, int nbins, double* partials,
+// Shell sums of a half spectrum: out (3 nbins doubles) = [sum of |F|^2 / N^3, sum of
+// 2 pi |n| / L, modes] per shell; scratch holds spectrum_scratch(n, nbins) doubles.
+size_t spectrum_scratch(int n, int nbins);
+cudaError_t launch_spectrum_bins(const void* spec, int n, double L, int nbins, double* scratch, double* out,
                                  cudaStream_t st);
 
 } // namespace lat
