@@ -247,19 +247,19 @@ lat_status configure_kernel(lat_handle* h, int variant, int ty, int zr, int dept
         return take(cfg, 5);
     }
     if (variant == 0 && h->esize == 4) {
-        // FP32: x tiles one warp wide unless they leave too many lanes of the
-        // warp empty. A row of one tile wants 17 lanes (64^3, 16 lanes: 13.1 us per
-        // step against 12.2 of variant 2; 68^3, 17 lanes: 14.4 against 16.5), a
-        // row of several 21 (160^3, 20 lanes: 42.1 against 41.8; 168^3, 21 lanes:
-        // 45.2 against 46.5; 384^3, 32 lanes: 298 against 435). Tiles of 16 rows
-        // with two planes in flight where the lanes are full or the row is one
-        // tile (512^3: 685 us, 8 rows 718; 100^3: 17.7, 17.8), else 8 rows with
-        // three, two blocks to an SM: with empty lanes a block moves fewer bytes
-        // per barrier (200^3: 62 against 64 us, 464^3: 579 against 592, 496^3:
-        // 700 against 710, 704^3: 2050 against 2138).
+        // FP32: tiles one warp wide where they fill enough of the warps' lanes. Whole
+        // rows (N <= 128) from 56 on (48^3: 10.2 us per step against 9.7 of variant
+        // 2, 56^3: 10.8 against 12.9, 100^3: 15.7 against 19.8); rows cut into x tiles
+        // from 21 lanes a tile on (160^3, 20 lanes: 42.1 against 41.8; 168^3, 21
+        // lanes: 45.2 against 46.5; 384^3, 32 lanes: 298 against 435). Tiles of 16
+        // rows with two planes in flight where the lanes are full or the row is one
+        // tile (512^3: 685 us, 8 rows 718), else 8 rows with three, two blocks to an
+        // SM: with empty lanes a block moves fewer bytes per barrier (200^3: 62
+        // against 64 us, 464^3: 579 against 592, 496^3: 700 against 710, 704^3: 2050
+        // against 2138).
         const int q = n / 4, nxt = (q + 31) / 32;
         MarchConfig cfg;
-        if (q / nxt >= (nxt == 1 ? 17 : 21)) {
+        if (nxt == 1 ? n >= 56 : q / nxt >= 21) {
             const bool tall = nxt == 1 || q == 32 * nxt;
             if (xw_config(n, 4, tall ? 16 : 8, 0, tall ? 2 : 3, &cfg) && fits(cfg)) return take(cfg, 5);
         }

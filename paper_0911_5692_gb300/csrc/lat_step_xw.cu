@@ -9,25 +9,42 @@ namespace lat {
 
 namespace {
 
-// The compiled instance of a tile height and prefetch depth, or null.
+// The compiled instance for a side, tile height and prefetch depth. FP32 sides of
+// at most 128 take whole rows in 16-row tiles with two planes in flight: without
+// the edge warp, and with two pairs of rows to a warp up to N = 64, a step is
+// 1.1 us (100^3: 16.8 -> 15.7) to 1.6 us (64^3: 12.6 -> 11.0) shorter.
+struct XWInst {
+    const void* fn = nullptr;
+    size_t smem = 0;
+    int threads = 0;
+};
 template <typename T>
-const void* xw_fn(int ty, int depth, size_t* smem)
+XWInst xw_inst(int n, int ty, int depth)
 {
-#define LAT_XW_CASE(TT, DD)                                 \
-    if (ty == TT && depth == DD) {                          \
-        *smem = xw::XW<T, TT, DD, false>::SMEM;             \
-        return (const void*)xw::step_xw_kernel<T, TT, DD, false>; \
+#define LAT_XW_CASE(TT, DD, SS)                                        \
+    {                                                                  \
+        typedef xw::XW<T, TT, DD, false, SS> F;                        \
+        return XWInst{(const void*)xw::step_xw_kernel<T, TT, DD, false, SS>, F::SMEM, F::THREADS}; \
     }
-    LAT_XW_CASE(16, 1) LAT_XW_CASE(16, 2)
-    if constexpr (sizeof(T) == 4) { LAT_XW_CASE(16, 3) LAT_XW_CASE(8, 2) LAT_XW_CASE(8, 3) }
-    else { LAT_XW_CASE(8, 1) LAT_XW_CASE(4, 1) }
+    if constexpr (sizeof(T) == 4) {
+        if (ty == 16 && depth == 2 && n <= 64) LAT_XW_CASE(16, 2, 16)
+        if (ty == 16 && depth == 2 && n <= 128) LAT_XW_CASE(16, 2, 32)
+        if (ty == 16 && depth == 3) LAT_XW_CASE(16, 3, 0)
+        if (ty == 8 && depth == 2) LAT_XW_CASE(8, 2, 0)
+        if (ty == 8 && depth == 3) LAT_XW_CASE(8, 3, 0)
+    } else {
+        if (ty == 8 && depth == 1) LAT_XW_CASE(8, 1, 0)
+        if (ty == 4 && depth == 1) LAT_XW_CASE(4, 1, 0)
+    }
+    if (ty == 16 && depth == 1) LAT_XW_CASE(16, 1, 0)
+    if (ty == 16 && depth == 2) LAT_XW_CASE(16, 2, 0)
 #undef LAT_XW_CASE
-    return nullptr;
+    return XWInst{};
 }
 
-const void* xw_kernel(int esize, int ty, int depth, size_t* smem)
+XWInst xw_inst(int esize, int n, int ty, int depth)
 {
-    return esize == 4 ? xw_fn<float>(ty, depth, smem) : xw_fn<double>(ty, depth, smem);
+    return esize == 4 ? xw_inst<float>(n, ty, depth) : xw_inst<double>(n, ty, depth);
 }
 
 } // namespace
@@ -39,18 +56,19 @@ bool xw_config(int n, int elem_bytes, int ty, int zr, int depth, MarchConfig* cf
     // second plane in flight takes the 512^3 FP32 step from 843 to 685 us and the
     // 256^3 step from 114 to 98; a third changes them by less than the runs differ)
     int d = depth;
-    size_t smem = 0;
-    const void* fn = nullptr;
-    if (d > 0) fn = xw_kernel(elem_bytes, tyv, d, &smem);
+    XWInst I;
+    if (d > 0) I = xw_inst(elem_bytes, n, tyv, d);
     else
         for (int dd : {2, 1})
-            if ((fn = xw_kernel(elem_bytes, tyv, dd, &smem))) {
+            if ((I = xw_inst(elem_bytes, n, tyv, dd)).fn) {
                 d = dd;
                 break;
             }
+    const void* fn = I.fn;
+    const size_t smem = I.smem;
     if (!fn || smem > 227 * 1024 - 2048) return false;
     const int vw = 16 / elem_bytes, nxt = (n / vw + 31) / 32;
-    const int threads = (tyv / 2 + 2) * 32;
+    const int threads = I.threads;
     if (allow_dynamic_smem(fn, smem) != cudaSuccess) return false;
     int occ = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, threads, smem) != cudaSuccess || occ < 1) return false;
@@ -90,8 +108,7 @@ template <typename T>
 cudaError_t launch_step_xw(const Bufs<T>& b, const Model& M, DevScalars* sc, double* partials, const MarchConfig& cfg,
                            cudaStream_t st)
 {
-    size_t smem = 0;
-    const void* fn = xw_fn<T>(cfg.ty, cfg.depth, &smem);
+    const void* fn = xw_inst<T>(M.n, cfg.ty, cfg.depth).fn;
     if (!fn) return cudaErrorInvalidValue;
     xw::SlabRun R{0, 0, nullptr};
     void* args[] = {(void*)&b, (void*)&M, (void*)&sc, (void*)&partials, (void*)&R};

@@ -59,17 +59,25 @@ namespace xw {
 
 enum { kPair, kAhead, kEdge, kIdle };   // warp roles
 
-template <typename T, int TY, int D, bool SLAB>
+// SW = 0: x tiles of up to 32 vectors and an edge warp. SW = 8, 16 or 32: rows of
+// one tile of at most SW vectors, 32 / SW pairs of rows to a warp; the row's ends
+// are each other's neighbours, reached by a shuffle, and there is no edge warp.
+template <typename T, int TY, int D, bool SLAB, int SW = 0>
 struct XW {
     typedef typename PK<T>::P P;
     static constexpr int RF = D + 2, RP = D + 1;       // field and momentum plane slots
     static constexpr int NP = PK<T>::NP;
     static constexpr int VW = 2 * NP;                  // elements per 16-byte vector
-    static constexpr int W = 32 * VW;                  // tile width: one warp of vectors
+    static constexpr bool EDGE = SW == 0;
+    static constexpr int LW = EDGE ? 32 : SW;          // lanes of a row
+    static constexpr int RPW = 32 / LW;                // pairs of rows to a warp
+    static constexpr int W = LW * VW;                  // tile width
     static constexpr int ROWS = TY + 3;                // staged rows
-    static constexpr int PAIRS = TY / 2;               // warps that own two rows each
-    static constexpr int THREADS = (PAIRS + 2) * 32;   // and the look-ahead and edge warps
-    static_assert(TY % 2 == 0 && ROWS <= 32, "row pairs; the edge warp has a lane per row");
+    static constexpr int PAIRS = TY / 2;               // pairs of owned rows
+    static constexpr int PWARPS = PAIRS / RPW;         // warps that own them
+    static constexpr int THREADS = (PWARPS + (EDGE ? 2 : 1)) * 32;   // and the look-ahead and edge warps
+    static_assert(TY % 2 == 0 && PAIRS % RPW == 0, "row pairs");
+    static_assert(!EDGE || ROWS <= 32, "the edge warp has a lane per row");
     // shared memory, in elements: the field ring [slot][field][ROWS][W], the
     // momentum ring [slot][field][TY + 1][W], the new fields of each pair's first
     // row and of the look-ahead row [buf][field][PAIRS + 1][W]; then the edge
@@ -82,7 +90,7 @@ struct XW {
     static constexpr uint32_t EF = ROWS * 4, ESF = 2 * EF;
     static constexpr uint32_t EPF = TY, ESP = 2 * EPF;
     static constexpr uint32_t EF0 = G0 + 2 * BUFG, EP0 = EF0 + RF * ESF, EG0 = EP0 + RP * ESP;
-    static constexpr uint32_t END = EG0 + 2 * 2 * TY;
+    static constexpr uint32_t END = EDGE ? EG0 + 2 * 2 * TY : EF0;
     static constexpr size_t SMEM = (sizeof(T) * (size_t)END + 15) / 16 * 16;
 
     struct Ctx {
@@ -92,6 +100,7 @@ struct XW {
         bool act;                        // this lane holds a vector of the tile
         uint32_t offF, offP, offG;       // this thread's vector of its (first) row: field, momentum, new-field planes
         uint32_t rowg, rowlo, rowhi;     // global offsets in a plane: its (first) row; the halo rows (look-ahead warp)
+        int lx, sl, sr;                  // its vector in the row; SW: the lanes of the neighbouring vectors
         int row, lane, z0, nz;           // its (first) row in the staged tile
         int zb;                          // SLAB: stored plane of the run's z = 0
         uint32_t ey, eyp;                // edge warp: offsets in a plane of its staged row and of owned row lane + 1
@@ -119,6 +128,16 @@ struct XW {
             const P z = mk2(T(0), T(0));
 #pragma unroll
             for (int r = 0; r < 2; r++) g[0][r] = g[1][r] = vd[r] = vi[r] = z;
+        }
+        __device__ __forceinline__ void add(const Acc& b)
+        {
+#pragma unroll
+            for (int r = 0; r < 2; r++) {
+                g[0][r] = add2(g[0][r], b.g[0][r]);
+                g[1][r] = add2(g[1][r], b.g[1][r]);
+                vd[r] = add2(vd[r], b.vd[r]);
+                vi[r] = add2(vi[r], b.vi[r]);
+            }
         }
     };
 
@@ -148,7 +167,7 @@ struct XW {
             }
         } else if constexpr (ROLE == kAhead) {
             T* d = C.S + slot * SLOTF + C.offF;
-            T* lo = C.S + slot * SLOTF + C.lane * VW;
+            T* lo = C.S + slot * SLOTF + C.lx * VW;
             if (C.act) {
                 cp_async16(lo, C.f0 + zoff + C.rowlo);
                 cp_async16(lo + FIELDF, C.f1 + zoff + C.rowlo);
@@ -261,9 +280,15 @@ struct XW {
                 P(&c)[NP] = Q.c[f][r];
                 // the neighbours in x of the vector's ends: the next lanes', or the
                 // tile's edge values (a predicated load, no branch on the lane)
-                const T left = ld_shared_if(C.lane == 0, Ec + f * EF + r * 4, __shfl_up_sync(0xffffffffu, hi2(c[NP - 1]), 1));
-                const T right = ld_shared_if(C.lane == C.last, Ec + f * EF + r * 4 + 1,
-                                             __shfl_down_sync(0xffffffffu, lo2(c[0]), 1));
+                T left, right;
+                if constexpr (EDGE) {
+                    left = ld_shared_if(C.lane == 0, Ec + f * EF + r * 4, __shfl_up_sync(0xffffffffu, hi2(c[NP - 1]), 1));
+                    right = ld_shared_if(C.lane == C.last, Ec + f * EF + r * 4 + 1,
+                                         __shfl_down_sync(0xffffffffu, lo2(c[0]), 1));
+                } else {
+                    left = __shfl_sync(0xffffffffu, hi2(c[NP - 1]), C.sl);
+                    right = __shfl_sync(0xffffffffu, lo2(c[0]), C.sr);
+                }
                 T d[VW];
                 xdiff<T>(c, right, d);
                 const T dl = s_sub(lo2(c[0]), left);
@@ -329,8 +354,10 @@ struct XW {
 #pragma unroll
                     for (int r = 0; r < R; r++) {
                         P(&q)[NP] = Q.g[f][r];
-                        const T right = ld_shared_if(C.lane == C.last, EGr + f * TY + r,
-                                                     __shfl_down_sync(0xffffffffu, lo2(q[0]), 1));
+                        T right;
+                        if constexpr (EDGE)
+                            right = ld_shared_if(C.lane == C.last, EGr + f * TY + r, __shfl_down_sync(0xffffffffu, lo2(q[0]), 1));
+                        else right = __shfl_sync(0xffffffffu, lo2(q[0]), C.sr);
                         T d[VW];
                         xdiff<T>(q, right, d);
 #pragma unroll
@@ -439,27 +466,79 @@ struct XW {
             if (k + 2 > C.nz) break;
         }
     }
+
+    // March planes C.z0 .. C.z0 + C.nz - 1 of the tile of rows y0 .. y0 + ty - 1 (ty
+    // even) and vectors q0 .. q0 + qn - 1. `first`: no earlier run of this block is
+    // still reading the ring.
+    static __device__ __forceinline__ void march(Ctx& C, int warp, int q0, int qn, int y0, int ty, bool first, Acc& A)
+    {
+        const int n = C.n;
+        const bool ahead = warp == PWARPS;
+        C.lane = threadIdx.x & 31;
+        C.lx = C.lane % LW;
+        C.ty = ty;
+        C.last = qn - 1;
+        const int pair = warp * RPW + C.lane / LW;
+        C.act = EDGE ? C.lx < qn : C.lx < qn && (ahead ? C.lane < LW : 2 * pair < ty);
+        C.row = ahead ? ty + 1 : 2 * pair + 1;
+        if constexpr (!EDGE) {
+            C.sl = C.lane - C.lx + (C.lx == 0 ? qn - 1 : C.lx - 1);
+            C.sr = C.lane - C.lx + (C.lx + 1 >= qn ? 0 : C.lx + 1);
+        }
+        C.offF = (uint32_t)C.row * W + C.lx * VW;
+        C.offP = (uint32_t)(C.row - 1) * W + C.lx * VW;
+        C.offG = (uint32_t)((C.row - 1) / 2) * W + C.lx * VW;
+        const int x0 = q0 * VW, x1 = x0 + qn * VW;
+        const uint32_t xg = x0 + C.lx * VW;
+        C.rowg = (uint32_t)wrapn(y0 + C.row - 1, n) * n + xg;
+        C.rowlo = (uint32_t)wrapn(y0 - 1, n) * n + xg;
+        C.rowhi = (uint32_t)wrapn(y0 + ty + 1, n) * n + xg;
+        if constexpr (EDGE) {
+            C.ey = (uint32_t)wrapn(y0 - 1 + min(C.lane, ty + 2), n) * n;
+            C.eyp = (uint32_t)wrapn(y0 + min(C.lane, ty - 1), n) * n;
+            // edge columns (periodic in x)
+            C.exl = (uint32_t)(x0 == 0 ? n - 1 : x0 - 1);
+            C.exr = (uint32_t)(x1 == n ? 0 : x1);
+            C.exr1 = (uint32_t)(x1 + 1 >= n ? x1 + 1 - n : x1 + 1);
+        }
+        // the previous segment's last plane is read by every thread before the
+        // prologue refills the ring
+        if (!first) __syncthreads();
+        if (ahead) run<kAhead>(C, A);
+        else if (EDGE && warp == PWARPS + 1) run<kEdge>(C, A);
+        else if (2 * warp * RPW < ty) run<kPair>(C, A);
+        else run<kIdle>(C, A);
+    }
+
+    // the four sums of this thread in the element type (1/beta and 1/2 are powers
+    // of two, exact)
+    static __device__ __forceinline__ void totals(const Acc& A, bool quartic, T (&v)[kSums])
+    {
+        v[0] = (lo2(A.g[0][0]) + hi2(A.g[0][0])) + (lo2(A.g[0][1]) + hi2(A.g[0][1]));
+        v[1] = (lo2(A.g[1][0]) + hi2(A.g[1][0])) + (lo2(A.g[1][1]) + hi2(A.g[1][1]));
+        v[2] = ((lo2(A.vd[0]) + hi2(A.vd[0])) + (lo2(A.vd[1]) + hi2(A.vd[1]))) * site_vsum_factor<T>(quartic);
+        v[3] = T(0.5) * ((lo2(A.vi[0]) + hi2(A.vi[0])) + (lo2(A.vi[1]) + hi2(A.vi[1])));
+    }
 };
 
-template <typename T, int TY, int D, bool SLAB>
-__global__ void __launch_bounds__(XW<T, TY, D, SLAB>::THREADS, TY <= 8 ? 2 : 1)
+template <typename T, int TY, int D, bool SLAB, int SW = 0>
+__global__ void __launch_bounds__(XW<T, TY, D, SLAB, SW>::THREADS, XW<T, TY, D, SLAB, SW>::THREADS <= 192 ? 2 : 1)
     step_xw_kernel(Bufs<T> B, Model M, DevScalars* sc, double* partials, SlabRun R)
 {
-    typedef XW<T, TY, D, SLAB> F;
-    constexpr int VW = F::VW, W = F::W;
+    typedef XW<T, TY, D, SLAB, SW> F;
+    constexpr int VW = F::VW;
     __shared__ double red[32 * kSums];
     extern __shared__ __align__(16) unsigned char smem_raw[];
     typename F::Ctx C;
     C.S = reinterpret_cast<T*>(smem_raw);
     const int warp = threadIdx.x >> 5;
-    C.lane = threadIdx.x & 31;
 
     // groups of nxt blocks: the x tiles of one y tile, marching the same
     // (y tile, z plane) units
     const int n = M.n;
     C.n = n;
     C.nn = (uint32_t)n * n;
-    const int nxt = (n / VW + 31) / 32, nyt = (n + TY - 1) / TY;
+    const int nxt = F::EDGE ? (n / VW + 31) / 32 : 1, nyt = (n + TY - 1) / TY;
     const int ngroups = gridDim.x / nxt;
     const int grp = blockIdx.x / nxt, xt = blockIdx.x - grp * nxt;
     TileWalk walk(nyt, ngroups, grp, SLAB ? R.nz : n);
@@ -469,13 +548,6 @@ __global__ void __launch_bounds__(XW<T, TY, D, SLAB>::THREADS, TY <= 8 ? 2 : 1)
     // tiles; lanes past the tile's last vector stage and store nothing
     const int Q = n / VW, cut = Q % 4 == 0 ? 4 : Q % 2 == 0 ? 2 : 1;
     const int q0 = xt * (Q / cut) / nxt * cut, qn = (xt + 1) * (Q / cut) / nxt * cut - q0;
-    const int x0 = q0 * VW, x1 = x0 + qn * VW;
-    C.last = qn - 1;
-    C.act = C.lane < qn;
-    // edge columns (periodic in x)
-    C.exl = (uint32_t)(x0 == 0 ? n - 1 : x0 - 1);
-    C.exr = (uint32_t)(x1 == n ? 0 : x1);
-    C.exr1 = (uint32_t)(x1 + 1 >= n ? x1 + 1 - n : x1 + 1);
 
     chain_begin();
     if (sc->status != LAT_OK) return;
@@ -495,7 +567,6 @@ __global__ void __launch_bounds__(XW<T, TY, D, SLAB>::THREADS, TY <= 8 ? 2 : 1)
     C.dtcf2 = mk2(C.K.dtcf, C.K.dtcf);
     typename F::Acc A;
     A.zero();
-
     C.zb = 0;
     int yt;
     for (bool first = true; walk.run(yt, C.z0, C.nz); first = false) {
@@ -519,33 +590,19 @@ __global__ void __launch_bounds__(XW<T, TY, D, SLAB>::THREADS, TY <= 8 ? 2 : 1)
         }
         walk.took(C.nz);
         const int y0 = 2 * (yt * (n / 2) / nyt), ty = 2 * ((yt + 1) * (n / 2) / nyt) - y0;
-        C.ty = ty;
-        const bool ahead = warp == F::PAIRS;
-        C.row = ahead ? ty + 1 : 2 * warp + 1;
-        C.offF = (uint32_t)C.row * W + C.lane * VW;
-        C.offP = (uint32_t)(C.row - 1) * W + C.lane * VW;
-        C.offG = (uint32_t)((C.row - 1) / 2) * W + C.lane * VW;
-        const uint32_t xg = x0 + C.lane * VW;
-        C.rowg = (uint32_t)wrapn(y0 + C.row - 1, n) * n + xg;
-        C.rowlo = (uint32_t)wrapn(y0 - 1, n) * n + xg;
-        C.rowhi = (uint32_t)wrapn(y0 + ty + 1, n) * n + xg;
-        C.ey = (uint32_t)wrapn(y0 - 1 + min(C.lane, ty + 2), n) * n;
-        C.eyp = (uint32_t)wrapn(y0 + min(C.lane, ty - 1), n) * n;
-        // the previous segment's last plane is read by every thread before the
-        // prologue refills the ring
-        if (!first) __syncthreads();
-        if (warp == F::PAIRS + 1) F::template run<kEdge>(C, A);
-        else if (ahead) F::template run<kAhead>(C, A);
-        else if (2 * warp < ty) F::template run<kPair>(C, A);
-        else F::template run<kIdle>(C, A);
+        if constexpr (F::EDGE) {
+            F::march(C, warp, q0, qn, y0, ty, first, A);
+        } else {   // a lane's pair of rows may lie past this tile's last
+            typename F::Acc S;
+            S.zero();
+            F::march(C, warp, q0, qn, y0, ty, first, S);
+            if (C.act) A.add(S);
+        }
     }
+    if (F::EDGE && (int)(threadIdx.x & 31) >= qn) A.zero();   // nothing in this lane
 
-    if (!C.act) A.zero();   // nothing in this lane
-    T v[kSums] = {(lo2(A.g[0][0]) + hi2(A.g[0][0])) + (lo2(A.g[0][1]) + hi2(A.g[0][1])),
-                  (lo2(A.g[1][0]) + hi2(A.g[1][0])) + (lo2(A.g[1][1]) + hi2(A.g[1][1])),
-                  ((lo2(A.vd[0]) + hi2(A.vd[0])) + (lo2(A.vd[1]) + hi2(A.vd[1]))) *
-                      site_vsum_factor<T>(C.K.quartic),
-                  T(0.5) * ((lo2(A.vi[0]) + hi2(A.vi[0])) + (lo2(A.vi[1]) + hi2(A.vi[1])))};
+    T v[kSums];
+    F::totals(A, C.K.quartic, v);
     if constexpr (SLAB) finish_block_sums(M, sc, partials, v, red, R.sums_out);
     else finish_block(M, sc, partials, v, red, true);
 }
