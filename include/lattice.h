@@ -514,7 +514,7 @@ typedef struct lat_batch lat_batch;
 /* Create `count` members from params[0..count-1] (all of one precision; each
  * member owns its buffers), bound to cuda_stream. The launch shape comes from
  * the process's autotuner cache for this set of sizes and precision, else a
- * default. LAT_EINVAL for mixed precisions or a bad member (its lat_create
+ * default (FP32 members of sides up to 128: whole rows in blocks of 256 threads). LAT_EINVAL for mixed precisions or a bad member (its lat_create
  * status is returned), LAT_EUNSUPPORTED if a member size fits no block shape or
  * a member has the 27-point stencil or expansion = 2. */
 lat_status lat_batch_create(const lat_params* params, int count, void* cuda_stream, lat_batch** out);
@@ -536,14 +536,16 @@ lat_status lat_batch_sync(lat_batch* b);
 /* Autotune the launch shape: time `steps` steps for each candidate of block
  * size (128 .. 1024), tile-height cap (32, 16, 8, 4; each member takes the
  * largest tile height up to the cap that divides its side and fits the block)
- * and prefetch depth (1 or 2 planes in flight ahead of the computed one) on the
+ * and prefetch depth (1 or 2 planes in flight ahead of the computed one), and the
+ * whole-row blocks of 256 threads where they serve every member, on the
  * ensemble itself, keep the fastest and cache it for this process per (sizes,
  * precision); ensembles created later with the same sizes and precision start
  * with it. Member states are saved before and restored after. Synchronises. */
 lat_status lat_batch_tune(lat_batch* b, int steps);
 
 /* The tile height (y rows per work unit) each member is stepped with:
- * ty (host, one int32 per member, in creation order). */
+ * ty (host, one int32 per member, in creation order). The whole-row blocks cut a
+ * side into tiles of an uneven number of pairs of rows: 2 for every member. */
 lat_status lat_batch_tile_heights(lat_batch* b, int32_t* ty);
 
 /* The launch shape in use (the block shape the paper picks by trial, Sec. II.C

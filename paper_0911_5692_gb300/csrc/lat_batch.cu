@@ -4,10 +4,12 @@
 // time and returns to the host every step).
 //
 // All (lattice, y tile, z plane) work of one step is laid out in one list,
-// weighted by sites, and cut into one contiguous range per resident block, so
+// weighted by its cost, and cut into one contiguous share per resident block, so
 // every block does the same amount of work whatever the member sizes. A block
-// marches its ranges with the plane-ring segment of lat_march.cuh, writes one
-// partial sum per range, and waits at a grid barrier: a counter and a generation
+// marches its ranges with the plane loop of lat_xw.cuh over whole rows (FP32
+// members of sides up to 128; 64 members of sides 32 to 96: 145 us per step) or the
+// plane-ring segment of lat_march.cuh (206 us there), writes one partial sum per
+// range, and waits at a grid barrier: a counter and a generation
 // word in device memory, with a wait bounded by the global timer (a block that
 // gives up sets LAT_ETIMEOUT and every block leaves at its next barrier, so a
 // broken launch returns an error instead of hanging). After the barrier every
@@ -31,6 +33,7 @@
 
 #include "lat_internal.h"
 #include "lat_march.cuh"
+#include "lat_xw.cuh"
 
 namespace lat {
 
@@ -67,87 +70,139 @@ __device__ __forceinline__ unsigned long long gtime()
 }
 
 // Grid-wide barrier with a bounded wait. Returns false (in every thread) if
-// this or another block gave up.
+// this or another block gave up. The arrival releases the block's writes and the
+// wait acquires the others' (each block's threads through the block barriers).
 __device__ bool grid_barrier(BatchCtl* ctl, unsigned int nblocks, unsigned long long timeout_ns)
 {
     __shared__ int ok;
     __syncthreads();
     if (threadIdx.x == 0) {
-        volatile unsigned int* vgen = &ctl->gen;
-        volatile int* vst = &ctl->status;
-        const unsigned int g = *vgen;
-        __threadfence();
+        auto load = [](const unsigned int* p) {
+            unsigned int v;
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+            return v;
+        };
+        const unsigned int g = load(&ctl->gen);
         int res = 1;
-        if (atomicAdd(&ctl->count, 1u) == nblocks - 1u) {
+        if (take_ticket(&ctl->count) == nblocks - 1u) {
             ctl->count = 0u;
-            __threadfence();
-            atomicExch(&ctl->gen, g + 1u);
+            asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(&ctl->gen), "r"(g + 1u) : "memory");
         } else {
             const unsigned long long t0 = gtime();
-            while (*vgen == g) {
-                if (*vst != LAT_OK || gtime() - t0 > timeout_ns) {
+            while (load(&ctl->gen) == g) {
+                if (*(volatile int*)&ctl->status != LAT_OK || gtime() - t0 > timeout_ns) {
                     atomicExch(&ctl->status, LAT_ETIMEOUT);
                     res = 0;
                     break;
                 }
-                __nanosleep(64);
             }
         }
-        if (*vst != LAT_OK) res = 0;
-        __threadfence();
+        if (*(volatile int*)&ctl->status != LAT_OK) res = 0;
         ok = res;
     }
     __syncthreads();
     return ok != 0;
 }
 
-// A scalar block written by another block earlier in this launch, read through
-// L2 (a plain load could return a line this SM cached before it was rewritten).
-__device__ inline void load_scalars_cg(const DevScalars* src, DevScalars& dst)
-{
-    static_assert(sizeof(DevScalars) % 8 == 0, "scalar block is copied in 8-byte words");
-    const unsigned long long* s = reinterpret_cast<const unsigned long long*>(src);
-    unsigned long long* d = reinterpret_cast<unsigned long long*>(&dst);
-    for (int i = 0; i < (int)(sizeof(DevScalars) / 8); i++) d[i] = __ldcg(s + i);
-}
-
-// Fold member l's range partials of one step (fixed order, warp 0) and advance
-// its scalars from `before`; result in `after` (thread 0).
+// Member BL's scalars at the start of a step into `cur`, by the whole block: from
+// those it started the step before with (`before`) and that step's range partials
+// (`part`, null at the first step of a launch: `before` as it is). Warp 1 forms
+// what does not depend on the sums while warp 0 folds the partials
+// (lat_common.cuh: the update takes about 2 us so, against 8 in one thread, in
+// every block and for every member it works on).
 template <typename T>
-__device__ __noinline__ void member_scalars(const BatchLat<T>& BL, const double* part, const DevScalars& before,
-                               DevScalars& after)
+__device__ void member_scalars(const BatchLat<T>& BL, const double* part, const DevScalars* before, DevScalars& cur)
 {
-    if (threadIdx.x >= 32) return;
-    double v[kSums] = {0.0, 0.0, 0.0, 0.0};
-    for (int s = BL.seg_begin + (int)threadIdx.x; s < BL.seg_end; s += 32)
-#pragma unroll
-        for (int k = 0; k < kSums; k++) v[k] += __ldcg(part + (size_t)s * kSums + k);
-#pragma unroll
-    for (int k = 0; k < kSums; k++)
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_down_sync(0xffffffffu, v[k], o);
-    if (threadIdx.x == 0) {
-        const Model& M = BL.M;
-        const double S[kSums] = {v[0] * M.inv_dx2 * M.inv_sites, v[1] * M.inv_dx2 * M.inv_sites, v[2] * M.inv_sites,
-                                 v[3] * M.inv_sites};
-        load_scalars_cg(&before, after);
-        advance_scalars(M, after, S, true);
+    __shared__ ScalePre pre;
+    const int warp = threadIdx.x >> 5, helper = blockDim.x > 32 ? 1 : 0;
+    __syncthreads();   // every thread is done with the previous member's scalars
+    if (warp == helper) {
+        scalars_to_shared(cur, before);
+        __syncwarp();
+        if (part) scale_pre_warp(BL.M, cur, pre, true);
+    }
+    double raw = 0.0;
+    if (part && warp == 0)
+        raw = warp_fold_partials(part + (size_t)BL.seg_begin * kSums, BL.seg_end - BL.seg_begin, 0, 1);
+    __syncthreads();
+    if (part) {
+        if (warp == 0) scale_finish_warp(BL.M, cur, pre, raw);
+        __syncthreads();
     }
 }
 
+// The block's four sums into row `s` of the step's partials.
+template <typename A>
+__device__ __forceinline__ void range_partials(const A v[kSums], double* red, double* pk, int s)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const TreeSum<A> r = warp_sum4(v);
+    if (lane < kSums) r.store(red, warp, lane);
+    __syncthreads();
+    if (warp == 0) {
+        const double t = warp_fold4<A>(red, block_warps());
+        if (lane < kSums) pk[(size_t)s * kSums + lane] = t;
+    }
+}
+
+// One range of a member whose rows are whole tiles of at most SW vectors (FP32, N
+// <= 128): the plane loop of the single-lattice step (lat_xw.cuh).
+template <typename F>
+__device__ __forceinline__ void rows_range(const BatchLat<float>& BL, const DevScalars& cur, const BatchSeg& g, float* S,
+                                           float (&v)[kSums])
+{
+    constexpr int TY = F::PAIRS * 2;
+    const int n = BL.M.n, nyt = (n + TY - 1) / TY;
+    const bool par = (cur.step & 1) != 0;
+    typename F::Ctx C;
+    C.S = S;
+    C.n = n;
+    C.nn = (uint32_t)n * n;
+    C.zb = 0;
+    C.z0 = g.z0;
+    C.nz = g.nz;
+    C.f0 = BL.buf[par ? 4 : 0];
+    C.f1 = BL.buf[par ? 5 : 1];
+    C.p0 = BL.buf[par ? 6 : 2];
+    C.p1 = BL.buf[par ? 7 : 3];
+    C.of0 = BL.buf[par ? 0 : 4];
+    C.of1 = BL.buf[par ? 1 : 5];
+    C.op0 = BL.buf[par ? 2 : 6];
+    C.op1 = BL.buf[par ? 3 : 7];
+    C.K = site_coefs<float>(&cur, BL.M.beta);
+    C.dtcl2 = mk2(C.K.dtcl, C.K.dtcl);
+    C.dtcf2 = mk2(C.K.dtcf, C.K.dtcf);
+    typename F::Acc A;
+    A.zero();
+    const int y0 = 2 * (g.yt * (n / 2) / nyt), ty = 2 * ((g.yt + 1) * (n / 2) / nyt) - y0;
+    // the block's barriers since its last range have passed every reader of the ring
+    F::march(C, threadIdx.x >> 5, 0, n / 4, y0, ty, true, A);
+    if (!C.act) A.zero();
+    F::totals(A, C.K.quartic, v);
+}
+// blocks of eight warps, seven of them with pairs of rows: 14, 28 or 56 rows to a
+// tile by the vectors of a row
+typedef xw::XW<float, 14, 2, false, 32> Rows32;
+typedef xw::XW<float, 28, 2, false, 16> Rows16;
+typedef xw::XW<float, 56, 2, false, 8> Rows8;
+constexpr int kRowThreads = 256, kRowSide = 128;
+static_assert(Rows32::THREADS == kRowThreads && Rows16::THREADS == kRowThreads && Rows8::THREADS == kRowThreads, "");
+constexpr size_t kRowSmem = Rows32::SMEM > Rows16::SMEM ? (Rows32::SMEM > Rows8::SMEM ? Rows32::SMEM : Rows8::SMEM)
+                                                        : (Rows16::SMEM > Rows8::SMEM ? Rows16::SMEM : Rows8::SMEM);
+int row_height(int n) { return n <= 32 ? 56 : n <= 64 ? 28 : 14; }
+
 // sc: two scalar slots per member ([2 l + slot]); slot 0 holds the scalars at
 // the start of the launch, slot (k & 1) those at the start of step k.
-// part: [2][nsegs][kSums]; cta: range table offsets per block.
-template <typename T, int MAXT, bool SPLIT>
-__global__ void __launch_bounds__(MAXT, MAXT <= 256 ? 3 : (MAXT <= 512 ? 2 : 1)) batch_kernel(const BatchLat<T>* __restrict__ lats,
-                                                     const BatchSeg* __restrict__ segs, const int* __restrict__ cta,
-                                                     int nsegs, DevScalars* sc, double* part, BatchCtl* ctl, int nsteps,
-                                                     int nlat, unsigned int extra, unsigned long long timeout_ns)
+// part: [2][nsegs][kSums]; cta: range table offsets per block. `range` marches one
+// range: (member, its scalars, range, ring, sums out, whether it is the block's first).
+template <typename T, typename Range>
+__device__ __forceinline__ void batch_steps(const BatchLat<T>* __restrict__ lats, const BatchSeg* __restrict__ segs,
+                                            const int* __restrict__ cta, int nsegs, DevScalars* sc, double* part,
+                                            BatchCtl* ctl, int nsteps, int nlat, unsigned int extra,
+                                            unsigned long long timeout_ns, T* S, Range range)
 {
     __shared__ double red[32 * kSums];
     __shared__ DevScalars cur;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    T* const S = reinterpret_cast<T*>(smem_raw);
     const int sb = cta[blockIdx.x], se = cta[blockIdx.x + 1];
     // `extra` > 0 only for the barrier self-test: the barrier then waits for
     // arrivals that never come and every block leaves when its wait runs out
@@ -164,49 +219,14 @@ __global__ void __launch_bounds__(MAXT, MAXT <= 256 ? 3 : (MAXT <= 512 ? 2 : 1))
             const BatchSeg g = segs[s];
             const BatchLat<T>& BL = lats[g.l];
             if (g.l != last_l) {
-                __syncthreads();   // every thread is done with the previous member's scalars
-                if (k == 0) {
-                    if (threadIdx.x == 0) cur = sc[2 * g.l];
-                } else {
-                    DevScalars after;
-                    member_scalars(BL, pprev, sc[2 * g.l + ((k - 1) & 1)], after);
-                    if (threadIdx.x == 0) {
-                        cur = after;
-                        if ((int)blockIdx.x == BL.owner) sc[2 * g.l + (k & 1)] = after;
-                    }
-                }
-                __syncthreads();
+                member_scalars(BL, k > 0 ? pprev : nullptr, sc + 2 * g.l + (k > 0 ? (k - 1) & 1 : 0), cur);
+                if (k > 0 && threadIdx.x < 32 && (int)blockIdx.x == BL.owner) scalars_from_shared(sc + 2 * g.l + (k & 1), cur);
                 last_l = g.l;
             }
-            double bs[kSums] = {0.0, 0.0, 0.0, 0.0};
-            if (cur.status == LAT_OK) {
-                const bool par = (cur.step & 1) != 0;
-                MarchLattice<T> L;
-                L.f0 = BL.buf[par ? 4 : 0];
-                L.f1 = BL.buf[par ? 5 : 1];
-                L.p0 = BL.buf[par ? 6 : 2];
-                L.p1 = BL.buf[par ? 7 : 3];
-                L.of0 = BL.buf[par ? 0 : 4];
-                L.of1 = BL.buf[par ? 1 : 5];
-                L.op0 = BL.buf[par ? 2 : 6];
-                L.op1 = BL.buf[par ? 3 : 7];
-                L.n = BL.M.n;
-                L.ty = BL.ty;
-                L.depth = BL.depth;
-                L.K = site_coefs<T>(&cur, BL.M.beta);
-                L.periodic = true;
-                L.zbase = 0;
-                MarchSums<T> A;
-                A.zero();
-                march_segment<T, SPLIT>(L, g.yt, g.z0, g.nz, S, A, s == sb);
-                T v[kSums];
-                A.totals(L.K.quartic, v);
-                block_reduce(v, red, bs);
-            }
-            if (threadIdx.x == 0)
-                for (int q = 0; q < kSums; q++) pk[(size_t)s * kSums + q] = bs[q];
+            T v[kSums] = {T(0), T(0), T(0), T(0)};
+            if (cur.status == LAT_OK) range(BL, cur, g, S, v, s == sb);
+            range_partials(v, red, pk, s);
         }
-        __threadfence();
         if (!grid_barrier(ctl, nblocks, timeout_ns)) return;
     }
     // scalars after the last step, stored by each member's owner
@@ -215,12 +235,66 @@ __global__ void __launch_bounds__(MAXT, MAXT <= 256 ? 3 : (MAXT <= 512 ? 2 : 1))
         for (int l = 0; l < nlat; l++) {
             const BatchLat<T>& BL = lats[l];
             if (BL.owner != (int)blockIdx.x) continue;
-            DevScalars after;
-            member_scalars(BL, plast, sc[2 * l + ((nsteps - 1) & 1)], after);
-            if (threadIdx.x == 0) sc[2 * l + (nsteps & 1)] = after;
-            __syncthreads();
+            member_scalars(BL, plast, sc + 2 * l + ((nsteps - 1) & 1), cur);
+            if (threadIdx.x < 32) scalars_from_shared(sc + 2 * l + (nsteps & 1), cur);
         }
     }
+}
+
+template <typename T, int MAXT, bool SPLIT>
+__global__ void __launch_bounds__(MAXT, MAXT <= 256 ? 3 : (MAXT <= 512 ? 2 : 1))
+    batch_kernel(const BatchLat<T>* __restrict__ lats, const BatchSeg* __restrict__ segs, const int* __restrict__ cta,
+                 int nsegs, DevScalars* sc, double* part, BatchCtl* ctl, int nsteps, int nlat, unsigned int extra,
+                 unsigned long long timeout_ns)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    batch_steps<T>(lats, segs, cta, nsegs, sc, part, ctl, nsteps, nlat, extra, timeout_ns, reinterpret_cast<T*>(smem_raw),
+                   [](const BatchLat<T>& BL, const DevScalars& cur, const BatchSeg& g, T* S, T (&v)[kSums], bool first) {
+                       const bool par = (cur.step & 1) != 0;
+                       MarchLattice<T> L;
+                       L.f0 = BL.buf[par ? 4 : 0];
+                       L.f1 = BL.buf[par ? 5 : 1];
+                       L.p0 = BL.buf[par ? 6 : 2];
+                       L.p1 = BL.buf[par ? 7 : 3];
+                       L.of0 = BL.buf[par ? 0 : 4];
+                       L.of1 = BL.buf[par ? 1 : 5];
+                       L.op0 = BL.buf[par ? 2 : 6];
+                       L.op1 = BL.buf[par ? 3 : 7];
+                       L.n = BL.M.n;
+                       L.ty = BL.ty;
+                       L.depth = BL.depth;
+                       L.K = site_coefs<T>(&cur, BL.M.beta);
+                       L.periodic = true;
+                       L.zbase = 0;
+                       MarchSums<T> A;
+                       A.zero();
+                       march_segment<T, SPLIT>(L, g.yt, g.z0, g.nz, S, A, first);
+                       A.totals(L.K.quartic, v);
+                   });
+}
+
+// The same over whole rows (every member FP32 with N <= 128). One block of eight
+// warps to an SM: up to eight warps a thread may hold 255 registers, and the plane
+// loop, which needs about 200 here, spills none (nine warps or two blocks of five
+// are held to 168: 64 members of sides 32 to 96 then take 212 to 266 us per step,
+// so 145; the full-row kernel of lat_march.cuh, tuned, 206). Two blocks of four
+// warps measured 142 to 214 by which members shared an SM: two of the three plane
+// loops at once overflow the instruction cache.
+__global__ void __launch_bounds__(kRowThreads, 1)
+    batch_rows_kernel(const BatchLat<float>* __restrict__ lats, const BatchSeg* __restrict__ segs,
+                      const int* __restrict__ cta, int nsegs, DevScalars* sc, double* part, BatchCtl* ctl, int nsteps,
+                      int nlat, unsigned int extra, unsigned long long timeout_ns)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    batch_steps<float>(lats, segs, cta, nsegs, sc, part, ctl, nsteps, nlat, extra, timeout_ns,
+                       reinterpret_cast<float*>(smem_raw),
+                       [](const BatchLat<float>& BL, const DevScalars& cur, const BatchSeg& g, float* S, float (&v)[kSums],
+                          bool) {
+                           const int n = BL.M.n;
+                           if (n <= 32) rows_range<Rows8>(BL, cur, g, S, v);
+                           else if (n <= 64) rows_range<Rows16>(BL, cur, g, S, v);
+                           else rows_range<Rows32>(BL, cur, g, S, v);
+                       });
 }
 
 // Copy the scalar blocks between the members' handles and the batch slots:
@@ -257,14 +331,16 @@ struct BatchShape {
     int tycap = 32;       // largest tile height a member takes
     int depth = 1;        // planes in flight ahead of the one computed
     int maxt = 0;
+    bool rows = false;    // batch_rows_kernel
     size_t smem = 0;
     int blocks = 0;
-    std::vector<int> ty;
+    std::vector<int> ty;  // rows of a tile (batch_rows_kernel: rows that stay together)
 };
 
 std::mutex g_tune_mutex;
 struct TunedShape {
     int threads, tycap, depth;
+    bool rows = false;
 };
 std::map<std::string, TunedShape> g_tuned;   // (sizes, precision) -> the fastest shape timed
 
@@ -317,6 +393,28 @@ std::string tune_key(const lat_batch* b)
 // Tile heights (each member the largest of 32, 16, ... 1 that divides its side,
 // is at most tycap and fits the block), ring size for the prefetch depth and
 // resident blocks for a block size; false if some member does not fit.
+bool rows_shape(const lat_batch* b, BatchShape* out)
+{
+    BatchShape s;
+    s.threads = kRowThreads;
+    s.depth = 2;
+    s.rows = true;
+    s.smem = kRowSmem;
+    for (lat_handle* h : b->h) {
+        if (h->prec != 32 || h->p.n > kRowSide) return false;
+        s.ty.push_back(2);   // tiles of an uneven number of pairs of rows
+    }
+    const void* fn = (const void*)batch_rows_kernel;
+    if (allow_dynamic_smem(fn, s.smem) != cudaSuccess) return false;
+    int occ = 0, dev = 0, sms = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, s.threads, s.smem) != cudaSuccess || occ < 1) return false;
+    cudaGetDevice(&dev);
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return false;
+    s.blocks = occ * sms;
+    *out = s;
+    return true;
+}
+
 bool shape_for(const lat_batch* b, int threads, int tycap, int depth, BatchShape* out)
 {
     BatchShape s;
@@ -352,44 +450,58 @@ bool shape_for(const lat_batch* b, int threads, int tycap, int depth, BatchShape
     return true;
 }
 
-// Lay out the (member, y tile, z plane) work, weighted by sites, in one
-// contiguous range per block, and upload the tables.
+// Lay out the (member, y tile, z plane) work, weighted by its cost, in one
+// contiguous share per block, and upload the tables.
 template <typename T>
 lat_status build_tables(lat_batch* b, const BatchShape& s)
 {
     const int nl = b->count;
-    std::vector<double> w;          // weight of each (member, y tile) column of planes
-    long long total = 0;
-    for (int l = 0; l < nl; l++) total += (long long)b->h[l]->nsites;
-    const int G = std::max(1, std::min<int>(s.blocks, (int)(total / 512 + 1)));
+    // Cost of a plane of a tile, and of starting a range, in sites. The full-row
+    // kernel of lat_march.cuh: its sites. batch_rows_kernel: a plane takes nearly the
+    // same time whatever its tile holds (its barrier and the chain of operations), and
+    // a range starts with about three planes' worth of loads (64 members of sides 32
+    // to 96: 153 us per step weighted by sites, 145.5 so).
+    const double fixed = s.rows ? 4096.0 : 0.0, start_planes = s.rows ? 3.0 : 0.0;
+    auto plane_cost = [&](int n, int rows) { return (double)n * rows + fixed; };
+    auto tiles = [&](int l, int n) { return s.rows ? (n + row_height(n) - 1) / row_height(n) : n / s.ty[l]; };
+    auto rows_of = [&](int l, int n, int yt, int nyt) {
+        return s.rows ? 2 * ((yt + 1) * (n / 2) / nyt) - 2 * (yt * (n / 2) / nyt) : s.ty[l];
+    };
+    long long sites = 0;
+    double total = 0.0;
+    for (int l = 0; l < nl; l++) {
+        const int n = b->h[l]->p.n, nyt = tiles(l, n);
+        sites += (long long)b->h[l]->nsites;
+        for (int yt = 0; yt < nyt; yt++) total += (n + start_planes) * plane_cost(n, rows_of(l, n, yt, nyt));
+    }
+    const int G = std::max(1, std::min<int>(s.blocks, (int)(sites / 512 + 1)));
     std::vector<BatchSeg> segs;
     std::vector<int> cta(G + 1, 0);
     std::vector<BatchLat<T>> lats(nl);
-    // walk the planes in order, cutting at multiples of total / G sites
-    long long acc = 0;
+    // walk the planes in order, cutting at multiples of total / G
+    double acc = 0.0;
     int blk = 0;
     for (int l = 0; l < nl; l++) {
         lat_handle* h = b->h[l];
-        const int n = h->p.n, ty = s.ty[l];
+        const int n = h->p.n, nyt = tiles(l, n);
         lats[l].M = h->M;
         for (int i = 0; i < 8; i++) lats[l].buf[i] = (T*)h->buf[i];
-        lats[l].ty = ty;
+        lats[l].ty = s.ty[l];
         lats[l].depth = s.depth;
         lats[l].seg_begin = (int)segs.size();
-        const long long per_plane = (long long)n * ty;
-        for (int yt = 0; yt < n / ty; yt++) {
+        for (int yt = 0; yt < nyt; yt++) {
+            const double cp = plane_cost(n, rows_of(l, n, yt, nyt));
+            double start = start_planes * cp;   // paid by the tile's first range
             int z = 0;
             while (z < n) {
                 // planes this block can still take before its share is full
-                const long long bound = (long long)((double)total * (blk + 1) / G);
-                long long room = (bound - acc + per_plane - 1) / per_plane;
-                if (blk == G - 1) room = n;
-                if (room < 1) room = 1;
-                const int nz = (int)std::min<long long>(room, n - z);
+                const double room = (total * (blk + 1) / G - acc - start) / cp;
+                int nz = blk == G - 1 ? n - z : (int)std::min<double>(n - z, std::max(1.0, std::floor(room + 0.5)));
                 segs.push_back(BatchSeg{l, yt, z, nz});
-                acc += per_plane * nz;
+                acc += start + cp * nz;
+                start = 0.0;
                 z += nz;
-                while (blk < G - 1 && acc >= (long long)((double)total * (blk + 1) / G)) {
+                while (blk < G - 1 && acc >= total * (blk + 1) / G - 0.5 * cp) {
                     blk++;
                     cta[blk] = (int)segs.size();
                 }
@@ -419,10 +531,10 @@ lat_status build_tables(lat_batch* b, const BatchShape& s)
     return LAT_OK;
 }
 
-lat_status configure(lat_batch* b, int threads, int tycap, int depth)
+lat_status configure(lat_batch* b, const TunedShape& t)
 {
     BatchShape s;
-    if (!shape_for(b, threads, tycap, depth, &s)) return LAT_EUNSUPPORTED;
+    if (t.rows ? !rows_shape(b, &s) : !shape_for(b, t.threads, t.tycap, t.depth, &s)) return LAT_EUNSUPPORTED;
     return b->prec == 32 ? build_tables<float>(b, s) : build_tables<double>(b, s);
 }
 
@@ -436,7 +548,7 @@ cudaError_t launch_batch(lat_batch* b, int64_t nsteps, unsigned int extra = 0,
     if (e != cudaSuccess) return e;
     e = cudaMemsetAsync(b->dctl, 0, sizeof(BatchCtl), b->stream);
     if (e != cudaSuccess) return e;
-    const void* fn = batch_fn<T>(b->shape.maxt, b->split);
+    const void* fn = b->shape.rows ? (const void*)batch_rows_kernel : batch_fn<T>(b->shape.maxt, b->split);
     const BatchLat<T>* lats = (const BatchLat<T>*)b->dlats;
     int nsegs = b->nsegs, ns = (int)nsteps, nlat = nl;
     void* args[] = {(void*)&lats, (void*)&b->dsegs, (void*)&b->dcta, (void*)&nsegs, (void*)&b->dsc,
@@ -497,6 +609,10 @@ lat_status autotune(lat_batch* b, int steps)
 {
     const std::string key = tune_key(b);
     std::vector<TunedShape> cands;
+    {
+        BatchShape s;
+        if (rows_shape(b, &s)) cands.push_back({s.threads, s.tycap, s.depth, true});
+    }
     for (int depth : {1, 2})
         for (int t : {128, 192, 256, 320, 384, 448, 512, 640, 768, 1024}) {
             std::vector<std::vector<int>> seen;
@@ -532,7 +648,7 @@ lat_status autotune(lat_batch* b, int steps)
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     if (st == LAT_OK && (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess)) st = LAT_ECUDA;
     for (size_t c = 0; c < cands.size() && st == LAT_OK; c++) {
-        if (configure(b, cands[c].threads, cands[c].tycap, cands[c].depth) != LAT_OK) continue;
+        if (configure(b, cands[c]) != LAT_OK) continue;
         if (run_steps(b, 2) != LAT_OK) continue;   // warm-up and graph
         cudaEventRecord(e0, b->stream);
         lat_status rs = run_steps(b, steps);
@@ -567,7 +683,7 @@ lat_status autotune(lat_batch* b, int steps)
         std::lock_guard<std::mutex> lock(g_tune_mutex);
         g_tuned[key] = best;
     }
-    return configure(b, best.threads, best.tycap, best.depth);
+    return configure(b, best);
 }
 
 } // namespace
@@ -613,11 +729,13 @@ lat_status lat_batch_create(const lat_params* params, int count, void* cuda_stre
             auto it = g_tuned.find(tune_key(b));
             if (it != g_tuned.end()) tuned = it->second;
         }
-        if (tuned.threads) st = configure(b, tuned.threads, tuned.tycap, tuned.depth);
+        if (tuned.threads) st = configure(b, tuned);
         else {
-            st = LAT_EUNSUPPORTED;
-            for (int t : {256, 512, 384, 640, 768, 1024, 128})
-                if ((st = configure(b, t, 32, 1)) == LAT_OK) break;
+            st = configure(b, TunedShape{kRowThreads, 32, 2, true});
+            for (int t : {256, 512, 384, 640, 768, 1024, 128}) {
+                if (st == LAT_OK) break;
+                st = configure(b, TunedShape{t, 32, 1});
+            }
         }
     }
     if (st != LAT_OK) {
@@ -685,7 +803,7 @@ lat_status lat_batch_set_shape(lat_batch* b, int threads, int tycap, int depth)
     LAT_CUDA(cudaStreamSynchronize(b->stream));
     BatchShape s;
     if (!shape_for(b, threads, tycap, depth, &s)) return LAT_EUNSUPPORTED;
-    return configure(b, threads, tycap, depth);
+    return configure(b, TunedShape{threads, tycap, depth});
 }
 
 lat_status lat_batch_shape(lat_batch* b, int64_t out[4])
