@@ -103,8 +103,8 @@ typedef struct {
  * dt^2 (k_max^2 + m_eff^2) > 4 at the initial state, with k_max^2 the
  * stencil's largest lattice frequency squared: 12/dx^2 for 7 points, 92/(15 dx^2)
  * for 27). The fields start at zero; call lat_init_fields or lat_set_state.
- * A 27-point lattice runs on the plane-ring step kernel only (variant 2 of
- * lat_set_kernel). On error *out is NULL. */
+ * A 27-point lattice runs on the step kernels of variants 2 and 5 of
+ * lat_set_kernel. On error *out is NULL. */
 lat_status lat_create(const lat_params* params, void* cuda_stream, lat_handle** out);
 
 /* As lat_create, with caller-owned device buffers (e.g. torch tensors):
@@ -299,7 +299,7 @@ lat_status lat_save_checkpoint(lat_handle* h, void* dst, uint64_t bytes);
 lat_status lat_load_checkpoint(lat_handle* h, const void* src, uint64_t bytes);
 
 /* Choose the step kernel (all compute the same step): variant 0 = automatic
- * (FP32: 5 where the x tiles fill enough of a warp's lanes, N > 64 but for
+ * (FP32: 5 where the x tiles fill enough of a warp's lanes, N >= 56 but for
  * sides between 128 and 168; otherwise 4 where a row is 128 or more 16-byte
  * vectors, FP64 N >= 256, else 2 where it fits, else 4), 2 = z-march through a
  * shared-memory plane ring over full x rows, filled by per-thread asynchronous
@@ -307,12 +307,12 @@ lat_status lat_load_checkpoint(lat_handle* h, const void* src, uint64_t bytes);
  * with taller y tiles, 5 = x tiles of at most 32 vectors, a warp to every two
  * rows, with ty and depth compiled in (FP32: ty 16 with depth 1, 2, 3, ty 8 with
  * 2, 3; FP64: ty 16 with depth 1, 2, ty 8 and 4 with 1) and one warp that handles
- * the tile's x neighbours; any N (4 and 5: 7-point only; the 27-point variant 5:
- * N = 256, 512);
+ * the tile's x neighbours; any N (4: 7-point only). A 27-point lattice: 5 for
+ * N > 64 (ty 14 with depth 2, ty 16 with 1), automatic there but for FP64 sides of
+ * 72 and 80; otherwise 2;
  * ty = owned rows per tile, zr = planes per z-chunk, depth = planes prefetched
  * ahead, 0 = automatic. LAT_EINVAL for another variant; LAT_EUNSUPPORTED if the
- * variant cannot run this lattice (a 27-point lattice runs on variant 2 only;
- * ty, zr and depth apply to it as above). */
+ * variant cannot run this lattice. */
 lat_status lat_set_kernel(lat_handle* h, int variant, int ty, int zr, int depth);
 
 /* Autotune the step kernel (the paper finds its block size by trial and error,
@@ -321,7 +321,7 @@ lat_status lat_set_kernel(lat_handle* h, int variant, int ty, int zr, int depth)
  * time `steps` steps (1 <= steps <= 100000, after a warm-up of 32 that also
  * captures the graph) for every kernel shape that can run this lattice --
  * variants 2, 4 and 5 over tile heights and prefetch depths (the 27-point
- * stencil: variant 2 over tile heights and depths) -- on the lattice's own
+ * stencil: variants 2 and 5) -- on the lattice's own
  * state, which is saved before and put back after every candidate and at the
  * end; keep the fastest, and remember it for the process per (N, precision,
  * stencil, split storage, expansion), so that handles created later with the

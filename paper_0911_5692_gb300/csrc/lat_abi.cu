@@ -224,7 +224,11 @@ lat_status configure_kernel(lat_handle* h, int variant, int ty, int zr, int dept
     if (h->M.stencil == 27) {   // the 27-point Laplacian: its own kernels (variants 2 and 5)
         if (variant == 4) return LAT_EUNSUPPORTED;
         MarchConfig cfg;
-        if (variant == 5 || variant == 0) {   // x tiles one warp wide where an instance is compiled
+        // x tiles one warp wide (sides above 64), but for the two FP64 sides that the
+        // plane ring runs as fast (72^3 182 us per step on both, 80^3 227 against 234;
+        // 68^3 335 against 183, 88^3 329 against 289)
+        const bool ring = h->esize == 8 && n < 88 && n % 8 == 0;
+        if (variant == 5 || (variant == 0 && !ring)) {
             if (s27w_config(n, (int)h->esize, variant == 0 ? 0 : ty, variant == 0 ? 0 : zr, variant == 0 ? 0 : depth,
                             &cfg) &&
                 fits(cfg))
@@ -309,6 +313,7 @@ std::vector<TuneShape> tune_candidates(const lat_handle* h)
 {
     std::vector<TuneShape> c;
     if (h->M.stencil == 27) {
+        c.push_back({5, 14, 0, 2});
         c.push_back({5, 16, 0, 1});
         for (int ty : {16, 8, 4})
             for (int d : {1, 2}) c.push_back({2, ty, 0, d});

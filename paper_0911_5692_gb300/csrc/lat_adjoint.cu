@@ -158,7 +158,7 @@ __device__ void adj_finish(T acc[kSums], double* red, AdjScalars* as, const AdjC
             base[3] = bad;
         }
     };
-    if (!block_ticket(acc, red, partials, &as->ticket, load, []() {})) return;
+    if (!block_ticket<T>(acc, red, partials, &as->ticket, load, []() {})) return;
     const double raw = last_block_fold(partials, red);
     if (linear_tid() >= 32) return;
     // the adjoints of cL, cF, cdom, kappa

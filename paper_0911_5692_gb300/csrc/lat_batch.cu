@@ -136,7 +136,7 @@ template <typename A>
 __device__ __forceinline__ void range_partials(const A v[kSums], double* red, double* pk, int s)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const TreeSum<A> r = warp_sum4(v);
+    const TreeSum<A> r = warp_sum4<A>(v);
     if (lane < kSums) r.store(red, warp, lane);
     __syncthreads();
     if (warp == 0) {

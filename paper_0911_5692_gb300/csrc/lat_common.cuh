@@ -380,15 +380,12 @@ struct TreeSum<double> {
 // of sums a lane carries, so 6 additions take the place of 20. Every lane ends
 // with the total of sum (lane & 3).
 template <typename A>
-__device__ __forceinline__ TreeSum<A> warp_sum4(const A v[kSums])
+__device__ __forceinline__ TreeSum<A> warp_sum4(const TreeSum<A> v[kSums])
 {
     const int lane = linear_tid() & 31;
     const bool b0 = lane & 1, b1 = lane & 2;
-    TreeSum<A> k0, k1, s0, s1;
-    k0.init(b0 ? v[1] : v[0]);
-    k1.init(b0 ? v[3] : v[2]);
-    s0.init(b0 ? v[0] : v[1]);
-    s1.init(b0 ? v[2] : v[3]);
+    TreeSum<A> k0 = b0 ? v[1] : v[0], k1 = b0 ? v[3] : v[2];
+    const TreeSum<A> s0 = b0 ? v[0] : v[1], s1 = b0 ? v[2] : v[3];
     k0.add(s0.shfl_xor(1));
     k1.add(s1.shfl_xor(1));
     TreeSum<A> r = b1 ? k1 : k0;
@@ -396,6 +393,15 @@ __device__ __forceinline__ TreeSum<A> warp_sum4(const A v[kSums])
 #pragma unroll
     for (int o = 4; o < 32; o <<= 1) r.add(r.shfl_xor(o));
     return r;
+}
+
+template <typename A>
+__device__ __forceinline__ TreeSum<A> warp_sum4(const A v[kSums])
+{
+    TreeSum<A> t[kSums];
+#pragma unroll
+    for (int k = 0; k < kSums; k++) t[k].init(v[k]);
+    return warp_sum4<A>(t);
 }
 
 // The warps' totals over a block, by one warp: every lane ends with the total of
@@ -657,8 +663,9 @@ __device__ __forceinline__ unsigned int take_ticket(unsigned int* ticket)
 // on its way `meanwhile` (warp 1, or warp 0 itself in a block of one warp). True
 // in every thread of the block that finished last; `red` (32 kSums doubles) is
 // free again then. `before` runs on warp 1 ahead of the block's ticket.
-template <typename A, typename Before, typename Meanwhile>
-__device__ __forceinline__ bool block_ticket(const A v[kSums], double* red, double* partials, unsigned int* ticket,
+// V: the element type A or TreeSum<A>.
+template <typename A, typename V, typename Before, typename Meanwhile>
+__device__ __forceinline__ bool block_ticket(const V v[kSums], double* red, double* partials, unsigned int* ticket,
                                              Before before, Meanwhile meanwhile)
 {
     const int nblocks = gridDim.x * gridDim.y * gridDim.z;
@@ -667,7 +674,7 @@ __device__ __forceinline__ bool block_ticket(const A v[kSums], double* red, doub
     const int helper = nwarps > 1 ? 1 : 0;
     __shared__ unsigned int is_last;
     if (warp == helper) before();
-    const TreeSum<A> r = warp_sum4(v);
+    const TreeSum<A> r = warp_sum4<A>(v);
     if (lane < kSums) r.store(red, warp, lane);
     __syncthreads();
     if (warp == 0) {
@@ -704,15 +711,15 @@ __device__ __forceinline__ double last_block_fold(const double* partials, double
 // then the a' solve and coefficients for the next step. `advance` is false for
 // the sums-only pass that follows initialisation or a state upload. The
 // per-thread sums are float (FP32 kernels) or double.
-template <typename A>
-__device__ inline void finish_block(const Model& M, DevScalars* sc, double* partials, A v[kSums],
-                                    double* red, bool advance)
+template <typename A, typename V>
+__device__ inline void finish_block_sums_of(const Model& M, DevScalars* sc, double* partials, const V* v, double* red,
+                                            bool advance)
 {
     __shared__ DevScalars img;
     __shared__ ScalePre pre;
     // the scalar block is read before this block's ticket: only the last block,
     // when every other has taken its own, rewrites it
-    if (!block_ticket(v, red, partials, &sc->ticket, [&]() { scalars_to_shared(img, sc); },
+    if (!block_ticket<A>(v, red, partials, &sc->ticket, [&]() { scalars_to_shared(img, sc); },
                       [&]() { scale_pre_warp(M, img, pre, advance); }))
         return;
     const double raw = last_block_fold(partials, red);
@@ -720,6 +727,20 @@ __device__ inline void finish_block(const Model& M, DevScalars* sc, double* part
     scale_finish_warp(M, img, pre, raw);
     scalars_from_shared(sc, img);
     if (advance && img.log) scalars_from_shared(img.log + (img.step - img.log_base), img);
+}
+
+template <typename A>
+__device__ inline void finish_block(const Model& M, DevScalars* sc, double* partials, A v[kSums], double* red,
+                                    bool advance)
+{
+    finish_block_sums_of<A>(M, sc, partials, v, red, advance);
+}
+// the same from sums that carry their rounding errors
+template <typename A>
+__device__ inline void finish_block_trees(const Model& M, DevScalars* sc, double* partials, const TreeSum<A> v[kSums],
+                                          double* red, bool advance)
+{
+    finish_block_sums_of<A>(M, sc, partials, v, red, advance);
 }
 
 // As finish_block, for a domain that is part of a larger lattice (a z-slab):
@@ -730,7 +751,7 @@ template <typename A>
 __device__ inline void finish_block_sums(const Model& M, DevScalars* sc, double* partials, A v[kSums], double* red,
                                          double* sums_out)
 {
-    if (!block_ticket(v, red, partials, &sc->ticket, []() {}, []() {})) return;
+    if (!block_ticket<A>(v, red, partials, &sc->ticket, []() {}, []() {})) return;
     const double raw = last_block_fold(partials, red);
     const int tid = linear_tid();
     if (tid < kSums) sums_out[tid] = raw * (tid < 2 ? M.grad_scale : M.inv_sites);

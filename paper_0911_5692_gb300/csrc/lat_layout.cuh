@@ -1,8 +1,6 @@
-// lat_layout.cuh -- how the 7-point step kernel that marches x tiles one warp
-// wide (variant 5, lat_xw.cuh) shares the (y tile, z plane) units of one step
-// among its block groups. (The 27-point kernel of variant 5 keeps one even
-// share of the units in (tile, z) order: with its longer prologue this layout
-// measured slower there.)
+// lat_layout.cuh -- how the step kernels that march x tiles one warp wide (variant
+// 5, lat_xw.cuh and lat_step27w.cu) share the (y tile, z plane) units of one step
+// among their block groups.
 #pragma once
 
 namespace lat {

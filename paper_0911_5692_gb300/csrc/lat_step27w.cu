@@ -1,15 +1,28 @@
 // lat_step27w.cu -- the fused leapfrog step with the 27-point Laplacian of
-// Sec. II.C (Patra and Karttunen) over x tiles one warp wide, with the lattice
-// side N, the tile height TY and the prefetch depth D known at compile time
-// (variant 5 of the 27-point stencil).
+// Sec. II.C (Patra and Karttunen) over x tiles one warp wide, with the tile
+// height TY and the prefetch depth D known at compile time and the lattice side
+// taken at run time (variant 5 of the 27-point stencil).
 //
-// Tiles, ring and edge warp follow the 7-point kernel of lat_step_xw.cu: a tile
-// is W = 32 16-byte vectors wide and TY rows tall, warp r stages row r (0: the
-// halo row below, 1..TY: the owned rows, TY + 1: the look-ahead row, TY + 2: the
-// halo row above), and one more warp (the edge warp) stages the scalars of the
-// tile's x neighbours, columns x0 - 1, x0 + W and x0 + W + 1, and computes the
-// new fields of the boundary column x0 + W, rounded exactly as the next tile
-// computes its own first column.
+// Tiles, ring and layout follow the 7-point kernel of lat_xw.cuh: a tile is at most
+// W = 32 16-byte vectors wide (a row's vectors are shared evenly among its tiles)
+// and at most TY rows tall. Two warps serve each pair of neighbouring rows: the step
+// warp kicks and drifts it, the sum warp adds up the new fields one plane later.
+// One more warp stages the halo rows, kicks and drifts the look-ahead row, and,
+// where the row is cut into x tiles, stages the scalars of the tile's x neighbours
+// (columns x0 - 1 and the two right of the tile) and computes the new fields of
+// the boundary column right of the tile, rounded exactly as the next tile computes
+// its own first column. Rows of one tile reach their ends by a rotating shuffle.
+//
+// What bounds it. FP32: the instructions of a plane, about 500 per row of a warp
+// (990 per pair against some 1500 with one row per warp and 13 squared bonds per
+// site), issued by 15 warps; the copy itself would take 79 us of the 117 at 256^3.
+// One warp for both halves of a pair's work held 252 registers, two warps to a
+// scheduler, and waited on its own latencies (issue slots 43 % busy, 126 us at
+// 256^3, 913 at 512^3); the two halves in two warps of 128 registers overlap, with
+// the new fields through shared memory: 117 and 824 us. One row per warp took 149
+// and 1187. Sides that only the plane-ring kernel ran before: 100^3 42 -> 19 us,
+// 292^3 1690 -> 206, 384^3 699 -> 369, 1024^3 13.4 -> 6.4 ms. FP64 is bound by the
+// FP64 pipe: 256^3 4.07 -> 3.51 ms.
 //
 // Laplacian. In units of 1/(30 dx^2) the weights are 14 (6 faces), 3 (12 edges)
 // and 1 (8 corners). Per plane p and site, with differences taken from that
@@ -25,30 +38,32 @@
 // Every term is a sum of differences of neighbouring values (exact for
 // f = const + small). The x-shifted sums are formed by scalar operations that
 // write the halves of the packed pairs, so no register moves build shifted
-// pairs. Along z each field keeps two packed values per site in registers:
-// the pending sum of plane z, L_z = (q_{z-1} - 30 (C_z - C_{z-1})) + r_z, and
-// q_z (C_z is read again from the ring); plane z + 1's aggregate, formed once,
-// completes
+// pairs. Along z each field keeps three values per site in registers: C_z, the
+// pending sum of plane z, L_z = (q_{z-1} - 30 (C_z - C_{z-1})) + r_z, and q_z;
+// plane z + 1's aggregate, formed once, completes
 // Lap(z) = (L_z + 30 (C_{z+1} - C_z)) + q_{z+1} and starts L_{z+1}. Every site's
 // value depends only on its 3x3x3 neighbourhood, not on the tiling or the z
 // segments.
 //
 // Sums of the new fields for eq. scale: -<g Lap g> is the mean over sites of
-// sum_b w_b (g(x + b) - g(x))^2 over the 13 bonds a site owns (all with
-// dy >= 0; the three with dz = -1 counted from the site above, as bonds between
-// rows y (plane P + 1) and y + 1 (plane P)). Each bond is summed by the warp of
-// its lower row at the column of its left end, so the only x neighbour a lane
-// needs is on its right: the next lane's first site, or for lane 31 the
-// boundary column. Bonds between planes P and P + 1 are summed at plane P + 2
-// from a ring of new-field planes, after the barrier that completes both.
-//
-// The NXT = N / W x tiles of a y tile are taken by NXT consecutive blocks that
-// march the same (y tile, z plane) units, so the edge scalars lie in memory
-// lines the neighbouring blocks are reading too (L2 hits).
+// sum_b w_b (g(x + b) - g(x))^2 over the 13 bonds a site owns. Over the whole
+// lattice that is a sum over its unit cubes, and there the bond energies are
+// diagonal in the cube's eight sign patterns: 15 for a pattern odd in one
+// direction, 20 in two, 23 in three (each squared, over 8). With the patterns odd
+// in x taken first, and their y and z sums and differences multiplied out,
+//   8 E = 312 dx^2 - 32 (dx dx_y + dx dx_z) - 4 (dx dx_yz + dx_y dx_z)
+//         + 70 B^2 - 10 B B_z + 15 Z^2,
+// dx the x difference (dx_y, dx_z, dx_yz: of the next row, the next plane, both),
+// B = dy + dy(x + 1), Z the sum of the cube's four z differences. Differences are
+// still formed first. That is 8 products per site for 13 squared bonds, one
+// shuffle a row for four, and only g and dx of the row above (the next pair's
+// first row, from shared memory) besides the pair's own. The cube between planes P
+// and P + 1 is summed at plane P + 2, after the barrier that completes P + 1.
 #include <algorithm>
 
 #include "lat_async.cuh"
 #include "lat_kernels.h"
+#include "lat_layout.cuh"
 #include "lat_pairs.cuh"
 #include "lat_site.cuh"
 
@@ -57,100 +72,142 @@ namespace lat {
 namespace {
 
 constexpr unsigned kFull = 0xffffffffu;
-enum { kOwn, kAhead, kStage, kEdge };   // warp roles
+enum { kStep, kSum, kAhead, kIdle };   // warp roles
 
-template <int D>
-struct Ring27W {
-    static constexpr int RF = D == 1 ? 4 : 6;          // field plane slots (>= D + 3)
-    static constexpr int RP = D + 1;                   // momentum plane slots
-    static constexpr int GS = D == 1 ? 4 : 3;          // new-field plane slots (3 in use)
-    static constexpr int PERIOD = D == 1 ? 4 : 6;      // lcm(RF, RP, GS)
-    static_assert(RF >= D + 3 && GS >= 3 && PERIOD % RF == 0 && PERIOD % RP == 0 && PERIOD % GS == 0,
-                  "ring period");
-};
-
-template <typename T, int N, int TY, int D>
+// EDGE: rows cut into x tiles; otherwise a row is one tile.
+template <typename T, int TY, int D, bool EDGE>
 struct S27 {
     typedef typename PK<T>::P P;
-    static constexpr int RF = Ring27W<D>::RF, RP = Ring27W<D>::RP, GS = Ring27W<D>::GS;
-    static constexpr int PERIOD = Ring27W<D>::PERIOD;
+    // field and momentum plane slots: planes z and z + 1 and D in flight, plane z
+    // and D
+    static constexpr int RF = D + 2, RP = D + 1;
     static constexpr int NP = PK<T>::NP;
     static constexpr int VW = 2 * NP;                  // elements per 16-byte vector
     static constexpr int W = 32 * VW;                  // tile width: one warp of vectors
-    static constexpr int NXT = N / W;                  // x tiles per row
-    static constexpr int ROWS = TY + 3;                // staged rows (one warp each)
-    static constexpr int GR = TY + 1;                  // computed rows (owned + look-ahead)
-    static constexpr int THREADS = (ROWS + 1) * 32;    // and the edge warp
-    static_assert(N % W == 0 && N % TY == 0 && GR <= 32, "tile geometry");
+    static constexpr int ROWS = TY + 3;                // staged rows, at most
+    static constexpr int GR = TY + 1;                  // computed rows (owned + look-ahead), at most
+    static constexpr int PAIRS = TY / 2;               // pairs of owned rows, two warps each
+    static constexpr int THREADS = (2 * PAIRS + 1) * 32;
+    static_assert(TY % 2 == 0 && ROWS <= 32, "row pairs; a lane per row for the edge columns");
     // Shared memory, in elements. The field ring [slot][field][ROWS][RS] with a
-    // row stride one vector longer than the tile (the edge warp reads the last
+    // row stride one vector longer than the tile (the edge column reads the last
     // column of every row: the padding spreads those reads over the banks), the
-    // momentum ring [slot][field][GR][W], the new-field ring [slot][field][GR][W];
-    // then the edge scalars: fields [slot][field][ROWS][4] (x0 - 1, x0 + W,
-    // x0 + W + 1, unused), momenta at x0 + W [slot][field][GR], new fields at
-    // x0 + W [slot][field][GR].
+    // momentum ring [slot][field][GR][W], the new fields [buf][field][GR][W]; then
+    // the edge scalars: fields [slot][field][ROWS][4] (x0 - 1, x0 + W, x0 + W + 1, unused),
+    // momenta at x0 + W [slot][field][GR], new fields at x0 + W [buf][field][GR].
     static constexpr int RS = W + VW;
     static constexpr uint32_t FIELDF = ROWS * RS, SLOTF = 2 * FIELDF;
     static constexpr uint32_t FIELDP = GR * W, SLOTP = 2 * FIELDP;
     static constexpr uint32_t P0 = RF * SLOTF, G0 = P0 + RP * SLOTP;
     static constexpr uint32_t EF = ROWS * 4, ESF = 2 * EF;
     static constexpr uint32_t ESP = 2 * GR;
-    static constexpr uint32_t EF0 = G0 + GS * SLOTP, EP0 = EF0 + RF * ESF, EG0 = EP0 + RP * ESP;
-    static constexpr uint32_t END = EG0 + GS * ESP;
+    static constexpr uint32_t EF0 = G0 + 2 * SLOTP, EP0 = EF0 + RF * ESF, EG0 = EP0 + RP * ESP;
+    static constexpr uint32_t END = EDGE ? EG0 + 2 * ESP : EF0;
     static constexpr size_t SMEM = (sizeof(T) * (size_t)END + 15) / 16 * 16;
-    static constexpr uint32_t NN = (uint32_t)N * N;
 
     struct Ctx {
         T* S;
-        uint32_t offF, offP, rowg;
-        int rho, lane, z0, nz;
-        uint32_t ey, eyp;               // edge warp: the row of its staged lane and of computed row lane + 1
+        uint32_t nn;
+        int n, ty, last;                // side, owned rows of the tile (even), its last lane
+        bool act;                       // this lane holds a vector of the tile
+        uint32_t offF, offP;            // this thread's vector of its (first) row: field and momentum planes
+        uint32_t rowg, rowlo, rowhi;    // global offsets in a plane: its (first) row; the halo rows (look-ahead warp)
+        int row, lane, sl, sr, z0, nz;  // its (first) row in the staged tile; the lanes beside it
+        uint32_t ey, eyp;               // edge columns: the row of staged row `lane` and of computed row lane + 1
         uint32_t exl, exr, exr1;        // the three edge columns
         const T *f0, *f1, *p0, *p1;
         T *of0, *of1, *op0, *op1;
         SiteCoefs<T> K;
-        P Lz[2][NP], Qz[2][NP];              // per field: L_z and q_z (row warps)
-        T eL[2], eQ[2], eC[2];               // L_z, q_z and C_z at the boundary column (edge warp)
-        P wg[2], vd, vi;                     // sums of the new fields
     };
-
-    static __device__ __forceinline__ bool edge_warp(const Ctx& C) { return C.rho == ROWS; }
+    struct Acc {
+        P wg[2], vd, vi;                // sums of the new fields (sum warps)
+    };
+    // ring slots of one plane step: field planes k + 1 and the one that plane
+    // k - 1 left, momentum plane k and the one that k - 1 left; new-field buffer
+    struct Slots {
+        int fc, fp, fw, pc, pw, g;
+        __device__ __forceinline__ void next()
+        {
+            fw = fc;
+            fc = fp;
+            fp = fp + 1 == RF ? 0 : fp + 1;
+            pw = pc;
+            pc = pc + 1 == RP ? 0 : pc + 1;
+            g ^= 1;
+        }
+    };
+    // carried from plane to plane, for each field and row: L_z and q_z (step
+    // and look-ahead warps; C_z is read again from the ring); the new fields, x differences and B of the
+    // pair's rows (the row after the pair as row 2), with the new fields right of
+    // the vector (sum warps)
+    template <int R>
+    struct Col {
+        P L[2][R][NP], q[2][R][NP];
+    };
+    struct Cube {
+        P g[2][3][NP], B[2][2][NP];
+        T r[2][3];
+    };
+    // the boundary column (lane r - 1 for computed row r)
+    struct EdgeCol {
+        T L[2], q[2], c[2];
+    };
 
     // plane z0 + zrel of the fields into ring slot `slot`
     template <int ROLE>
-    static __device__ __forceinline__ void fetch_f(Ctx& C, int zrel, int slot)
+    static __device__ __forceinline__ void fetch_f(const Ctx& C, int zrel, int slot)
     {
-        const uint32_t zoff = (uint32_t)wrapn(C.z0 + zrel, N) * NN;
-        if constexpr (ROLE != kEdge) {
-            const uint32_t gi = zoff + C.rowg;
+        const uint32_t zoff = (uint32_t)wrapn(C.z0 + zrel, C.n) * C.nn;
+        if constexpr (ROLE == kStep) {
+            const T *a = C.f0 + zoff + C.rowg, *b = C.f1 + zoff + C.rowg;
             T* d = C.S + slot * SLOTF + C.offF;
-            cp_async16(d, C.f0 + gi);
-            cp_async16(d + FIELDF, C.f1 + gi);
-        } else if (C.lane < ROWS) {
-            const uint32_t gb = zoff + C.ey;
-            T* e = C.S + EF0 + slot * ESF + C.lane * 4;
-            cp_async_small<sizeof(T)>(e + 0, C.f0 + gb + C.exl);
-            cp_async_small<sizeof(T)>(e + 1, C.f0 + gb + C.exr);
-            cp_async_small<sizeof(T)>(e + 2, C.f0 + gb + C.exr1);
-            cp_async_small<sizeof(T)>(e + EF + 0, C.f1 + gb + C.exl);
-            cp_async_small<sizeof(T)>(e + EF + 1, C.f1 + gb + C.exr);
-            cp_async_small<sizeof(T)>(e + EF + 2, C.f1 + gb + C.exr1);
+            if (C.act) {
+                cp_async16(d, a);
+                cp_async16(d + RS, a + C.n);
+                cp_async16(d + FIELDF, b);
+                cp_async16(d + FIELDF + RS, b + C.n);
+            }
+        } else if constexpr (ROLE == kAhead) {
+            T* d = C.S + slot * SLOTF + C.offF;
+            T* lo = C.S + slot * SLOTF + C.lane * VW;
+            if (C.act) {
+                cp_async16(lo, C.f0 + zoff + C.rowlo);
+                cp_async16(lo + FIELDF, C.f1 + zoff + C.rowlo);
+                cp_async16(d, C.f0 + zoff + C.rowg);
+                cp_async16(d + FIELDF, C.f1 + zoff + C.rowg);
+                cp_async16(d + RS, C.f0 + zoff + C.rowhi);
+                cp_async16(d + FIELDF + RS, C.f1 + zoff + C.rowhi);
+            }
+            if (EDGE && C.lane < C.ty + 3) {
+                const uint32_t gb = zoff + C.ey;
+                T* e = C.S + EF0 + slot * ESF + C.lane * 4;
+                cp_async_small<sizeof(T)>(e + 0, C.f0 + gb + C.exl);
+                cp_async_small<sizeof(T)>(e + 1, C.f0 + gb + C.exr);
+                cp_async_small<sizeof(T)>(e + 2, C.f0 + gb + C.exr1);
+                cp_async_small<sizeof(T)>(e + EF + 0, C.f1 + gb + C.exl);
+                cp_async_small<sizeof(T)>(e + EF + 1, C.f1 + gb + C.exr);
+                cp_async_small<sizeof(T)>(e + EF + 2, C.f1 + gb + C.exr1);
+            }
         }
     }
-    // momenta of plane z0 + zrel for the computed rows, and at x0 + W (edge warp,
-    // lane r - 1 for row r)
+    // momenta of plane z0 + zrel for the computed rows, and at x0 + W
     template <int ROLE>
-    static __device__ __forceinline__ void fetch_p(Ctx& C, int zrel, int slot)
+    static __device__ __forceinline__ void fetch_p(const Ctx& C, int zrel, int slot)
     {
-        const uint32_t zoff = (uint32_t)wrapn(C.z0 + zrel, N) * NN;
-        if constexpr (ROLE != kEdge) {
-            if constexpr (ROLE != kStage) {
-                const uint32_t gi = zoff + C.rowg;
-                T* d = C.S + P0 + slot * SLOTP + C.offP;
-                cp_async16(d, C.p0 + gi);
-                cp_async16(d + FIELDP, C.p1 + gi);
+        const uint32_t zoff = (uint32_t)wrapn(C.z0 + zrel, C.n) * C.nn;
+        if constexpr (ROLE == kStep || ROLE == kAhead) {
+            const T *a = C.p0 + zoff + C.rowg, *b = C.p1 + zoff + C.rowg;
+            T* d = C.S + P0 + slot * SLOTP + C.offP;
+            if (C.act) {
+                cp_async16(d, a);
+                cp_async16(d + FIELDP, b);
+                if constexpr (ROLE == kStep) {
+                    cp_async16(d + W, a + C.n);
+                    cp_async16(d + FIELDP + W, b + C.n);
+                }
             }
-        } else if (C.lane < GR) {
+        }
+        if (EDGE && ROLE == kAhead && C.lane <= C.ty) {
             const uint32_t gb = zoff + C.eyp + C.exr;
             T* e = C.S + EP0 + slot * ESP + C.lane;
             cp_async_small<sizeof(T)>(e, C.p0 + gb);
@@ -158,58 +215,73 @@ struct S27 {
         }
     }
 
-    // x neighbours of this lane's vector: from the adjacent lanes, at the tile's
-    // ends the edge scalars (*el at x0 - 1, *er at x0 + W), read by those lanes
-    // only. Every lane calls this.
-    static __device__ __forceinline__ void xnb(const P (&v)[NP], const T* el, const T* er, int lane, T& l, T& r)
-    {
-        l = ld_shared_if(lane == 0, el, __shfl_up_sync(kFull, hi2(v[NP - 1]), 1));
-        r = ld_shared_if(lane == 31, er, __shfl_down_sync(kFull, lo2(v[0]), 1));
-    }
-
-    // The aggregates of one field at this lane's sites of row rho: centres c,
+    // The aggregates of one field at this lane's sites of its R rows: centres c,
     // q = 3 e + k and r = 14 e + 3 k. F: the field's plane in the ring, E: its
     // edge scalars. Every lane calls this.
-    static __device__ __forceinline__ void aggr(const Ctx& C, const T* F, const T* E, P (&c)[NP], P (&q)[NP],
-                                                P (&r)[NP])
+    template <int R>
+    static __device__ __forceinline__ void aggr(const Ctx& C, const T* F, const T* E, P (&c)[R][NP], P (&q)[R][NP],
+                                                P (&r)[R][NP])
     {
         const T* row = F + C.offF;
-        P m[NP], p[NP];
-        PK<T>::ld(row, c);
-        PK<T>::ld(row - RS, m);
-        PK<T>::ld(row + RS, p);
-        const T* e = E + C.rho * 4;
-        T cl, cr, ml, mr, pl, pr;
-        xnb(c, e, e + 1, C.lane, cl, cr);
-        xnb(m, e - 4, e - 3, C.lane, ml, mr);
-        xnb(p, e + 4, e + 5, C.lane, pl, pr);
-        P v[NP];
-        T cs[VW + 2], vs[VW + 2];
+        P up[NP], dn[NP], v[R][NP];
+        PK<T>::ld(row - RS, up);
+#pragma unroll
+        for (int i = 0; i < R; i++) PK<T>::ld(row + i * RS, c[i]);
+        PK<T>::ld(row + R * RS, dn);
+        // the column beside the tile's end that this lane is at, rows row - 1 ..
+        // row + R, and its y pairs
+        T ec[R + 2], ev[R];
+        const bool first = C.lane == 0, last = C.lane == C.last;
+        if constexpr (EDGE) {
+            const T* e = E + (C.row - 1) * 4 + (first ? 0 : 1);
+#pragma unroll
+            for (int i = 0; i < R + 2; i++) ec[i] = ld_shared_if(first || last, e + 4 * i, T(0));
+#pragma unroll
+            for (int i = 0; i < R; i++) ev[i] = s_add(s_sub(ec[i], ec[i + 1]), s_sub(ec[i + 2], ec[i + 1]));
+        }
+        // the y difference inside a pair serves both rows
 #pragma unroll
         for (int j = 0; j < NP; j++) {
-            v[j] = add2(sub2(m[j], c[j]), sub2(p[j], c[j]));
-            cs[1 + 2 * j] = lo2(c[j]);
-            cs[2 + 2 * j] = hi2(c[j]);
-            vs[1 + 2 * j] = lo2(v[j]);
-            vs[2 + 2 * j] = hi2(v[j]);
+            if constexpr (R == 2) {
+                const P in = sub2(c[1][j], c[0][j]);
+                v[0][j] = add2(sub2(up[j], c[0][j]), in);
+                v[1][j] = sub2(sub2(dn[j], c[1][j]), in);
+            } else {
+                v[0][j] = add2(sub2(up[j], c[0][j]), sub2(dn[j], c[0][j]));
+            }
         }
-        cs[0] = cl;
-        cs[VW + 1] = cr;
-        vs[0] = s_add(s_sub(ml, cl), s_sub(pl, cl));
-        vs[VW + 1] = s_add(s_sub(mr, cr), s_sub(pr, cr));
-        T dd[VW + 1];   // differences of consecutive sites
-#pragma unroll
-        for (int i = 0; i <= VW; i++) dd[i] = s_sub(cs[i + 1], cs[i]);
         const P two = mk2(T(2), T(2)), three = mk2(T(3), T(3)), fourteen = mk2(T(14), T(14));
 #pragma unroll
-        for (int j = 0; j < NP; j++) {
-            const int a = 1 + 2 * j, b = 2 + 2 * j;   // positions of the pair's sites in cs and vs
-            const P h = mk2(s_sub(dd[a], dd[a - 1]), s_sub(dd[b], dd[b - 1]));
-            const P t = mk2(s_add(vs[a - 1], vs[a + 1]), s_add(vs[b - 1], vs[b + 1]));
-            const P k = fma2(two, h, t);
-            const P eh = add2(h, v[j]);
-            q[j] = fma2(three, eh, k);
-            r[j] = fma2(fourteen, eh, mul2(three, k));
+        for (int i = 0; i < R; i++) {
+            T cs[VW + 2], vs[VW + 2];
+#pragma unroll
+            for (int j = 0; j < NP; j++) {
+                un2(c[i][j], cs[1 + 2 * j], cs[2 + 2 * j]);
+                un2(v[i][j], vs[1 + 2 * j], vs[2 + 2 * j]);
+            }
+            cs[0] = __shfl_sync(kFull, cs[VW], C.sl);
+            cs[VW + 1] = __shfl_sync(kFull, cs[1], C.sr);
+            vs[0] = __shfl_sync(kFull, vs[VW], C.sl);
+            vs[VW + 1] = __shfl_sync(kFull, vs[1], C.sr);
+            if constexpr (EDGE) {
+                cs[0] = first ? ec[i + 1] : cs[0];
+                vs[0] = first ? ev[i] : vs[0];
+                cs[VW + 1] = last ? ec[i + 1] : cs[VW + 1];
+                vs[VW + 1] = last ? ev[i] : vs[VW + 1];
+            }
+            T dd[VW + 1];   // differences of consecutive sites
+#pragma unroll
+            for (int x = 0; x <= VW; x++) dd[x] = s_sub(cs[x + 1], cs[x]);
+#pragma unroll
+            for (int j = 0; j < NP; j++) {
+                const int a = 1 + 2 * j, b = 2 + 2 * j;   // positions of the pair's sites in cs and vs
+                const P h = mk2(s_sub(dd[a], dd[a - 1]), s_sub(dd[b], dd[b - 1]));
+                const P t = mk2(s_add(vs[a - 1], vs[a + 1]), s_add(vs[b - 1], vs[b + 1]));
+                const P k = fma2(two, h, t);
+                const P eh = add2(h, v[i][j]);
+                q[i][j] = fma2(three, eh, k);
+                r[i][j] = fma2(fourteen, eh, mul2(three, k));
+            }
         }
     }
 
@@ -228,148 +300,140 @@ struct S27 {
         r = s_fma(T(14), eh, s_mul(T(3), k));
     }
 
-    // Edge warp: the aggregates at (x0 + W, row r) of one field's plane F (ring)
-    // with edge scalars E; the site's centre in *c.
-    static __device__ __forceinline__ void aggr_edge(const T* F, const T* E, int r, T& c, T& q, T& r_)
+    // The aggregates at (x0 + W, row r) of one field's plane F (ring) with edge
+    // scalars E; the site's centre in c.
+    static __device__ __forceinline__ void aggr_edge(const Ctx& C, const T* F, const T* E, int r, T& c, T& q, T& r_)
     {
-        const T* lc = F + r * RS + (W - 1);
+        const T* lc = F + r * RS + (C.last * VW + VW - 1);
         const T* e = E + r * 4;
         c = e[1];
         aggr1(lc[0], e[1], e[2], lc[-RS], e[-3], e[-2], lc[RS], e[5], e[6], q, r_);
     }
 
-    // Bonds of the new-field planes P (Gp) and P + 1 (Gu) at this lane's sites
-    // of owned row rho, and the potential sums of plane P. EGp, EGu: the
-    // boundary column of both planes. Every lane of an owned row calls this.
-    static __device__ __forceinline__ void bonds(Ctx& C, const T* Gp, const T* Gu, const T* EGp, const T* EGu)
+    // Takes the pair's new fields of plane P from G (the column right of the tile
+    // from EG) and, where SUM is set, adds the cubes between plane P - 1 (in H) and
+    // P, and the potential of plane P - 1; leaves plane P in H. Every lane calls
+    // this.
+    template <bool SUM>
+    static __device__ __forceinline__ void cubes(const Ctx& C, Acc& A, Cube& H, const T* G, const T* EG)
     {
-        P pz[2][NP];
+        const bool last = C.lane == C.last;
+        const T* gp = G + (C.row - 1) * W + C.lane * VW;
+        const T* ep = EG + (C.row - 1);
+        if constexpr (SUM) {
+#pragma unroll
+            for (int j = 0; j < NP; j++) {
+                site_vsum<T>(C.K, H.g[0][0][j], H.g[1][0][j], A.vd, A.vi);
+                site_vsum<T>(C.K, H.g[0][1][j], H.g[1][1][j], A.vd, A.vi);
+            }
+        }
 #pragma unroll
         for (int f = 0; f < 2; f++) {
-            const T* gp = Gp + f * FIELDP + C.offP;
-            const T* gu = Gu + f * FIELDP + C.offP;
-            P p0[NP], p1[NP], u0[NP], u1[NP];
-            PK<T>::ld(gp, p0);
-            PK<T>::ld(gp + W, p1);
-            PK<T>::ld(gu, u0);
-            PK<T>::ld(gu + W, u1);
-            const int eb = f * GR + C.rho - 1;
-            // right neighbours of element VW - 1; lane 31: the boundary column
-            const bool last = C.lane == 31;
-            const T p0e = ld_shared_if(last, EGp + eb, __shfl_down_sync(kFull, lo2(p0[0]), 1));
-            const T p1e = ld_shared_if(last, EGp + eb + 1, __shfl_down_sync(kFull, lo2(p1[0]), 1));
-            const T u0e = ld_shared_if(last, EGu + eb, __shfl_down_sync(kFull, lo2(u0[0]), 1));
-            const T u1e = ld_shared_if(last, EGu + eb + 1, __shfl_down_sync(kFull, lo2(u1[0]), 1));
-            // the rows shifted one site to the right
-            P p0R[NP], p1R[NP], u0R[NP], u1R[NP];
+            P g[3][NP], dx[3][NP], dp[3][NP], B[2][NP];
+            T re[3];
 #pragma unroll
-            for (int j = 0; j < NP; j++) {
-                const bool lastj = j == NP - 1;
-                p0R[j] = mk2(hi2(p0[j]), lastj ? p0e : lo2(p0[lastj ? j : j + 1]));
-                p1R[j] = mk2(hi2(p1[j]), lastj ? p1e : lo2(p1[lastj ? j : j + 1]));
-                u0R[j] = mk2(hi2(u0[j]), lastj ? u0e : lo2(u0[lastj ? j : j + 1]));
-                u1R[j] = mk2(hi2(u1[j]), lastj ? u1e : lo2(u1[lastj ? j : j + 1]));
+            for (int i = 0; i < 3; i++) PK<T>::ld(gp + f * FIELDP + i * W, g[i]);
+#pragma unroll
+            for (int i = 0; i < 3; i++) {
+                re[i] = __shfl_sync(kFull, lo2(g[i][0]), C.sr);
+                if constexpr (EDGE) re[i] = ld_shared_if(last, ep + f * GR + i, re[i]);
+                T d[VW];
+                xdiff<T>(g[i], re[i], d);
+#pragma unroll
+                for (int j = 0; j < NP; j++) dx[i][j] = mk2(d[2 * j], d[2 * j + 1]);
+                if constexpr (SUM) {
+                    xdiff<T>(H.g[f][i], H.r[f][i], d);
+#pragma unroll
+                    for (int j = 0; j < NP; j++) dp[i][j] = mk2(d[2 * j], d[2 * j + 1]);
+                }
             }
-            const P zero = mk2(T(0), T(0));
-            P a14 = zero, a3 = zero, a1 = zero;
+            // a + a(x + 1) of a vector whose right neighbour is e
+            auto xsum = [](const P(&a)[NP], T e, P(&o)[NP]) {
+                T s[VW + 1];
 #pragma unroll
-            for (int j = 0; j < NP; j++) {
-                const P c = p0[j];
-                P d;
-                // faces: (1,0,0) (0,1,0) (0,0,1)
-                d = sub2(p0R[j], c); a14 = fma2(d, d, a14);
-                d = sub2(p1[j], c);  a14 = fma2(d, d, a14);
-                d = sub2(u0[j], c);  a14 = fma2(d, d, a14);
-                // edges: (1,1,0) (-1,1,0) (1,0,1) (-1,0,1) (0,1,1), and (0,1,-1) from the site above
-                d = sub2(p1R[j], c);      a3 = fma2(d, d, a3);
-                d = sub2(p1[j], p0R[j]);  a3 = fma2(d, d, a3);
-                d = sub2(u0R[j], c);      a3 = fma2(d, d, a3);
-                d = sub2(u0[j], p0R[j]);  a3 = fma2(d, d, a3);
-                d = sub2(u1[j], c);       a3 = fma2(d, d, a3);
-                d = sub2(p1[j], u0[j]);   a3 = fma2(d, d, a3);
-                // corners: (1,1,1) (-1,1,1), and (1,1,-1) (-1,1,-1) from the site above
-                d = sub2(u1R[j], c);      a1 = fma2(d, d, a1);
-                d = sub2(u1[j], p0R[j]);  a1 = fma2(d, d, a1);
-                d = sub2(p1R[j], u0[j]);  a1 = fma2(d, d, a1);
-                d = sub2(p1[j], u0R[j]);  a1 = fma2(d, d, a1);
-                pz[f][j] = c;
+                for (int j = 0; j < NP; j++) un2(a[j], s[2 * j], s[2 * j + 1]);
+                s[VW] = e;
+#pragma unroll
+                for (int j = 0; j < NP; j++) o[j] = mk2(s_add(s[2 * j], s[2 * j + 1]), s_add(s[2 * j + 1], s[2 * j + 2]));
+            };
+#pragma unroll
+            for (int i = 0; i < 2; i++) {
+                P dy[NP];
+#pragma unroll
+                for (int j = 0; j < NP; j++) dy[j] = sub2(g[i + 1][j], g[i][j]);
+                xsum(dy, s_sub(re[i + 1], re[i]), B[i]);
             }
-            // this plane's bonds by weight, folded into the field's sum
-            C.wg[f] = fma2(mk2(T(14), T(14)), a14, fma2(mk2(T(3), T(3)), a3, add2(a1, C.wg[f])));
-        }
+            if constexpr (SUM) {
+                P dz[3][NP];
+                T de[3];
 #pragma unroll
-        for (int j = 0; j < NP; j++) site_vsum<T>(C.K, pz[0][j], pz[1][j], C.vd, C.vi);
-    }
-
-    // the top of every plane: wait for plane k + 1 (and its momenta), the
-    // barrier, then the prefetch of plane k + D + 1
-    template <int J, int ROLE>
-    static __device__ __forceinline__ void plane_top(Ctx& C, int k)
-    {
-        cp_async_wait(D - 1);
-        __syncthreads();
-        if (k + D <= C.nz) {
-            fetch_f<ROLE>(C, k + D + 1, (J + D + 2) % RF);
-            fetch_p<ROLE>(C, k + D, (J + D) % RP);
-        }
-        cp_async_commit();
-    }
-    // the prologue of a run: planes z0 - 1 .. z0 + D of the fields, z0 .. z0 + D - 1
-    // of the momenta, one commit group per plane step
-    template <int ROLE>
-    static __device__ __forceinline__ void prologue(Ctx& C)
-    {
-        fetch_f<ROLE>(C, -1, 0);
-        fetch_f<ROLE>(C, 0, 1);
-        fetch_f<ROLE>(C, 1, 2);
-        fetch_p<ROLE>(C, 0, 0);
-        cp_async_commit();
+                for (int i = 0; i < 3; i++) {
 #pragma unroll
-        for (int j = 1; j < D; j++) {
-            fetch_f<ROLE>(C, j + 1, j + 2);
-            fetch_p<ROLE>(C, j, j);
-            cp_async_commit();
+                    for (int j = 0; j < NP; j++) dz[i][j] = sub2(g[i][j], H.g[f][i][j]);
+                    de[i] = s_sub(re[i], H.r[f][i]);
+                }
+                const P zero = mk2(T(0), T(0));
+                P s0 = zero, s1 = zero, s2 = zero, b1 = zero, b2 = zero, z = zero;
+#pragma unroll
+                for (int i = 0; i < 2; i++) {
+                    P S[NP], Z[NP];
+#pragma unroll
+                    for (int j = 0; j < NP; j++) S[j] = add2(dz[i][j], dz[i + 1][j]);
+                    xsum(S, s_add(de[i], de[i + 1]), Z);
+#pragma unroll
+                    for (int j = 0; j < NP; j++) {
+                        const P d = dp[i][j], dn = dp[i + 1][j];
+                        s0 = fma2(d, d, s0);
+                        s1 = fma2(d, add2(dn, dx[i][j]), s1);
+                        s2 = fma2(d, dx[i + 1][j], fma2(dn, dx[i][j], s2));
+                        b1 = fma2(H.B[f][i][j], H.B[f][i][j], b1);
+                        b2 = fma2(H.B[f][i][j], B[i][j], b2);
+                        z = fma2(Z[j], Z[j], z);
+                    }
+                }
+                // this plane's cubes by weight (over 8), folded into the field's sum
+                auto w = [](double c) { return mk2(T(c), T(c)); };
+                P t = fma2(w(-0.5), s2, A.wg[f]);
+                t = fma2(w(-1.25), b2, t);
+                t = fma2(w(-4.0), s1, t);
+                t = fma2(w(1.875), z, t);
+                t = fma2(w(8.75), b1, t);
+                A.wg[f] = fma2(w(39.0), s0, t);
+            }
+#pragma unroll
+            for (int i = 0; i < 3; i++) {
+#pragma unroll
+                for (int j = 0; j < NP; j++) H.g[f][i][j] = g[i][j];
+                H.r[f][i] = re[i];
+            }
+#pragma unroll
+            for (int i = 0; i < 2; i++)
+#pragma unroll
+                for (int j = 0; j < NP; j++) H.B[f][i][j] = B[i][j];
         }
     }
 
-    // Edge warp, plane k: the boundary column x0 + W of computed row r = lane + 1.
-    template <int J>
-    static __device__ __forceinline__ void plane_edge(Ctx& C, int k)
+    // Plane k of the boundary column right of the tile at computed row r = lane + 1.
+    static __device__ __forceinline__ void plane_edge(const Ctx& C, const Slots& Z, EdgeCol& E)
     {
-        plane_top<J, kEdge>(C, k);
         const int r = C.lane + 1;
-        if (r > GR) return;
-        const T* Fm = C.S + (J % RF) * SLOTF;
-        const T* Fc = C.S + ((J + 1) % RF) * SLOTF;
-        const T* Fp = C.S + ((J + 2) % RF) * SLOTF;
-        const T* Em = C.S + EF0 + (J % RF) * ESF;
-        const T* Ec = C.S + EF0 + ((J + 1) % RF) * ESF;
-        const T* Ep = C.S + EF0 + ((J + 2) % RF) * ESF;
-        const T* Epc = C.S + EP0 + (J % RP) * ESP;
-        T* EGw = C.S + EG0 + (J % GS) * ESP;
-        if (J == 0 && k == 0) {   // the first plane of a run: L and q of planes z0 - 1 and z0
-#pragma unroll
-            for (int f = 0; f < 2; f++) {
-                T cm, qm, rm, cc, qc, rc;
-                aggr_edge(Fm + f * FIELDF, Em + f * EF, r, cm, qm, rm);
-                aggr_edge(Fc + f * FIELDF, Ec + f * EF, r, cc, qc, rc);
-                C.eL[f] = s_add(s_fma(T(-30), s_sub(cc, cm), qm), rc);
-                C.eQ[f] = qc;
-                C.eC[f] = cc;
-            }
-        }
+        if (r > C.ty + 1) return;
+        const T* Fp = C.S + Z.fp * SLOTF;
+        const T* Ep = C.S + EF0 + Z.fp * ESF;
+        const T* Epc = C.S + EP0 + Z.pc * ESP;
+        T* EGw = C.S + EG0 + Z.g * ESP;
         T cz[2], pn[2];
 #pragma unroll
         for (int f = 0; f < 2; f++) {
             T cp, qp, rp;
-            aggr_edge(Fp + f * FIELDF, Ep + f * EF, r, cp, qp, rp);
-            const T d = s_sub(cp, C.eC[f]);
-            const T lap = s_add(s_fma(T(30), d, C.eL[f]), qp);
-            pn[f] = s_fma(C.K.dtcl, lap, s_fma(C.K.dtcf, C.eC[f], Epc[f * GR + (r - 1)]));
-            C.eL[f] = s_add(s_fma(T(-30), d, C.eQ[f]), rp);
-            C.eQ[f] = qp;
-            cz[f] = C.eC[f];
-            C.eC[f] = cp;
+            aggr_edge(C, Fp + f * FIELDF, Ep + f * EF, r, cp, qp, rp);
+            const T d = s_sub(cp, E.c[f]);
+            const T lap = s_add(s_fma(T(30), d, E.L[f]), qp);
+            pn[f] = s_fma(C.K.dtcl, lap, s_fma(C.K.dtcf, E.c[f], Epc[f * GR + (r - 1)]));
+            E.L[f] = s_add(s_fma(T(-30), d, E.q[f]), rp);
+            E.q[f] = qp;
+            cz[f] = E.c[f];
+            E.c[f] = cp;
         }
         T g0, g1;
         site_kick_drift1<T>(C.K, cz[0], cz[1], pn[0], pn[1], g0, g1);
@@ -377,114 +441,216 @@ struct S27 {
         EGw[GR + (r - 1)] = g1;
     }
 
-    // Row warps, plane k: kick and drift of the computed rows, and the bonds of
-    // planes k - 2 and k - 1 (both written before the barrier) for the owned rows.
-    // ROLE (the same for the whole warp and the whole run): kOwn, kAhead (the
-    // look-ahead row, computed but not stored) or kStage (the halo rows, staged
-    // only).
-    template <int J, int ROLE>
-    static __device__ __forceinline__ void plane_rows(Ctx& C, int k)
+    // Plane k of a pair (R = 2; stored) or of the look-ahead row (R = 1): kick and
+    // drift.
+    template <int R>
+    static __device__ __forceinline__ void plane_rows(const Ctx& C, const Slots& Z, Col<R>& Q, int k)
     {
-        plane_top<J, ROLE>(C, k);
-        constexpr bool comp = ROLE != kStage;
-        constexpr bool own = ROLE == kOwn;
-        const T* Fm = C.S + (J % RF) * SLOTF;
-        const T* Fc = C.S + ((J + 1) % RF) * SLOTF;
-        const T* Fp = C.S + ((J + 2) % RF) * SLOTF;
-        const T* Pc = C.S + P0 + (J % RP) * SLOTP;
-        T* Gw = C.S + G0 + (J % GS) * SLOTP;
-        const T* Gm1 = C.S + G0 + ((J + GS - 1) % GS) * SLOTP;   // plane k - 1
-        const T* Gm2 = C.S + G0 + ((J + GS - 2) % GS) * SLOTP;   // plane k - 2
-        const T* Em = C.S + EF0 + (J % RF) * ESF;
-        const T* Ec = C.S + EF0 + ((J + 1) % RF) * ESF;
-        const T* Ep = C.S + EF0 + ((J + 2) % RF) * ESF;
-        const T* EGm1 = C.S + EG0 + ((J + GS - 1) % GS) * ESP;
-        const T* EGm2 = C.S + EG0 + ((J + GS - 2) % GS) * ESP;
-
-        if (comp) {
-            const P c30 = mk2(T(30), T(30)), cm30 = mk2(T(-30), T(-30));
-            if (J == 0 && k == 0) {   // the first plane of a run: L and q of planes z0 - 1 and z0
+        const T* Fc = C.S + Z.fc * SLOTF + C.offF;
+        const T* Fp = C.S + Z.fp * SLOTF;
+        const T* Pc = C.S + P0 + Z.pc * SLOTP + C.offP;
+        const T* Ep = C.S + EF0 + Z.fp * ESF;
+        T* Gw = C.S + G0 + Z.g * SLOTP + C.offP;
+        const P c30 = mk2(T(30), T(30)), cm30 = mk2(T(-30), T(-30));
+        const P dtcl2 = mk2(C.K.dtcl, C.K.dtcl), dtcf2 = mk2(C.K.dtcf, C.K.dtcf);
+        P pn[2][R][NP], cz[2][R][NP], g[2][R][NP];
 #pragma unroll
-                for (int f = 0; f < 2; f++) {
-                    P cm[NP], qm[NP], rm[NP], cc[NP], qc[NP], rc[NP];
-                    aggr(C, Fm + f * FIELDF, Em + f * EF, cm, qm, rm);
-                    aggr(C, Fc + f * FIELDF, Ec + f * EF, cc, qc, rc);
+        for (int f = 0; f < 2; f++) {
+            P cp[R][NP], qp[R][NP], rp[R][NP];
 #pragma unroll
-                    for (int j = 0; j < NP; j++) {
-                        C.Lz[f][j] = add2(fma2(cm30, sub2(cc[j], cm[j]), qm[j]), rc[j]);
-                        C.Qz[f][j] = qc[j];
-                    }
-                }
+            for (int i = 0; i < R; i++) {
+                PK<T>::ld(Pc + f * FIELDP + i * W, pn[f][i]);
+                PK<T>::ld(Fc + f * FIELDF + i * RS, cz[f][i]);
             }
-            P pn[2][NP], cz[2][NP];
-            const P dtcl2 = mk2(C.K.dtcl, C.K.dtcl), dtcf2 = mk2(C.K.dtcf, C.K.dtcf);
+            aggr<R>(C, Fp + f * FIELDF, Ep + f * EF, cp, qp, rp);
 #pragma unroll
-            for (int f = 0; f < 2; f++) {
-                P cp[NP], qp[NP], rp[NP], pv[NP];
-                PK<T>::ld(Fc + f * FIELDF + C.offF, cz[f]);   // C_z
-                aggr(C, Fp + f * FIELDF, Ep + f * EF, cp, qp, rp);
-                PK<T>::ld(Pc + f * FIELDP + C.offP, pv);
+            for (int i = 0; i < R; i++)
 #pragma unroll
                 for (int j = 0; j < NP; j++) {
-                    const P d = sub2(cp[j], cz[f][j]);
-                    const P lap = add2(fma2(c30, d, C.Lz[f][j]), qp[j]);
-                    pn[f][j] = fma2(dtcl2, lap, fma2(dtcf2, cz[f][j], pv[j]));
-                    C.Lz[f][j] = add2(fma2(cm30, d, C.Qz[f][j]), rp[j]);
-                    C.Qz[f][j] = qp[j];
+                    const P c = cz[f][i][j], d = sub2(cp[i][j], c);
+                    const P lap = add2(fma2(c30, d, Q.L[f][i][j]), qp[i][j]);
+                    pn[f][i][j] = fma2(dtcl2, lap, fma2(dtcf2, c, pn[f][i][j]));
+                    Q.L[f][i][j] = add2(fma2(cm30, d, Q.q[f][i][j]), rp[i][j]);
+                    Q.q[f][i][j] = qp[i][j];
                 }
-            }
-            P g[2][NP];
-            // potential part of the kick and the drift (lat_site.cuh)
-#pragma unroll
-            for (int j = 0; j < NP; j++) site_kick_drift<T>(C.K, cz[0][j], cz[1][j], pn[0][j], pn[1][j], g[0][j], g[1][j]);
-            if (own && k < C.nz) {
-                const uint32_t gi = (uint32_t)(C.z0 + k) * NN + C.rowg;
-                PK<T>::st(C.op0 + gi, pn[0]);
-                PK<T>::st(C.op1 + gi, pn[1]);
-                PK<T>::st(C.of0 + gi, g[0]);
-                PK<T>::st(C.of1 + gi, g[1]);
-            }
-            PK<T>::st(Gw + C.offP, g[0]);
-            PK<T>::st(Gw + FIELDP + C.offP, g[1]);
         }
-        if (own && k >= 2) bonds(C, Gm2, Gm1, EGm2, EGm1);
+        // potential part of the kick and the drift (lat_site.cuh)
+#pragma unroll
+        for (int i = 0; i < R; i++)
+#pragma unroll
+            for (int j = 0; j < NP; j++)
+                site_kick_drift<T>(C.K, cz[0][i][j], cz[1][i][j], pn[0][i][j], pn[1][i][j], g[0][i][j], g[1][i][j]);
+        if (R == 2 && k < C.nz && C.act) {
+            const uint32_t gi = (uint32_t)wrapn(C.z0 + k, C.n) * C.nn + C.rowg;
+#pragma unroll
+            for (int i = 0; i < R; i++) {
+                PK<T>::st_stream(C.op0 + gi + i * C.n, pn[0][i]);
+                PK<T>::st_stream(C.op1 + gi + i * C.n, pn[1][i]);
+                PK<T>::st_stream(C.of0 + gi + i * C.n, g[0][i]);
+                PK<T>::st_stream(C.of1 + gi + i * C.n, g[1][i]);
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < R; i++) {
+            PK<T>::st(Gw + i * W, g[0][i]);
+            PK<T>::st(Gw + FIELDP + i * W, g[1][i]);
+        }
     }
 
-    // planes k + J .. k + PERIOD - 1; false once the look-ahead plane is done
-    template <int J, int ROLE>
-    static __device__ __forceinline__ bool planes(Ctx& C, int k)
+    // One plane: 0, 1 or 2 planes of this run are behind it (2: or more).
+    template <int ROLE, int BEHIND, int R>
+    static __device__ __forceinline__ void plane(const Ctx& C, Acc& A, Slots& Z, Col<R>& Q, Cube& H, EdgeCol& E, int k)
     {
-        if constexpr (ROLE == kEdge) plane_edge<J>(C, k + J);
-        else plane_rows<J, ROLE>(C, k + J);
-        if (k + J + 1 > C.nz) return false;
-        if constexpr (J + 1 < PERIOD) return planes<J + 1, ROLE>(C, k);
-        else return true;
+        cp_async_wait(D - 1);
+        __syncthreads();
+        if ((ROLE == kStep || ROLE == kAhead) && k + D <= C.nz) {
+            fetch_f<ROLE>(C, k + D + 1, Z.fw);
+            fetch_p<ROLE>(C, k + D, Z.pw);
+        }
+        cp_async_commit();
+        if constexpr (ROLE == kSum && BEHIND > 0)
+            cubes<(BEHIND > 1)>(C, A, H, C.S + G0 + (Z.g ^ 1) * SLOTP, C.S + EG0 + (Z.g ^ 1) * ESP);
+        if constexpr (EDGE && ROLE == kAhead) plane_edge(C, Z, E);
+        if constexpr (ROLE == kStep || ROLE == kAhead) plane_rows<R>(C, Z, Q, k);
+        Z.next();
     }
+
+    // One run of planes: the prologue (planes z0 - 1 .. z0 + D of the fields,
+    // z0 .. z0 + D - 1 of the momenta, one commit group per plane step; C, L and q of
+    // the first plane into registers), then the planes, and the last cubes, between
+    // planes nz - 1 and nz (the look-ahead plane). Every role passes the same
+    // barriers.
     template <int ROLE>
-    static __device__ __forceinline__ void run(Ctx& C)
+    static __device__ __forceinline__ void run(const Ctx& C, Acc& A)
     {
-        prologue<ROLE>(C);
-        for (int k = 0; planes<0, ROLE>(C, k); k += PERIOD) {}
+        constexpr int R = ROLE == kStep ? 2 : 1;
+        fetch_f<ROLE>(C, -1, 0);
+        fetch_f<ROLE>(C, 0, 1);
+        fetch_f<ROLE>(C, 1, 2);
+        fetch_p<ROLE>(C, 0, 0);
+        cp_async_commit();
+#pragma unroll
+        for (int j = 1; j < D; j++) {
+            if (j <= C.nz) {
+                fetch_f<ROLE>(C, j + 1, j + 2);
+                fetch_p<ROLE>(C, j, j);
+            }
+            cp_async_commit();
+        }
+        cp_async_wait(D - 1);
+        __syncthreads();
+        Col<R> Q;
+        Cube H;
+        EdgeCol E;
+        if constexpr (ROLE == kStep || ROLE == kAhead) {
+            const P cm30 = mk2(T(-30), T(-30));
+            P cm[R][NP], c[R][NP], q[R][NP], r[R][NP];
+#pragma unroll
+            for (int f = 0; f < 2; f++) {
+                aggr<R>(C, C.S + f * FIELDF, C.S + EF0 + f * EF, cm, Q.q[f], r);
+                aggr<R>(C, C.S + SLOTF + f * FIELDF, C.S + EF0 + ESF + f * EF, c, q, r);
+#pragma unroll
+                for (int i = 0; i < R; i++)
+#pragma unroll
+                    for (int j = 0; j < NP; j++) {
+                        Q.L[f][i][j] = add2(fma2(cm30, sub2(c[i][j], cm[i][j]), Q.q[f][i][j]), r[i][j]);
+                        Q.q[f][i][j] = q[i][j];
+                    }
+            }
+        }
+        if constexpr (EDGE && ROLE == kAhead) {
+            const int r = min(C.lane, C.ty) + 1;
+#pragma unroll
+            for (int f = 0; f < 2; f++) {
+                T cm, qm, rm, cc, qc, rc;
+                aggr_edge(C, C.S + f * FIELDF, C.S + EF0 + f * EF, r, cm, qm, rm);
+                aggr_edge(C, C.S + SLOTF + f * FIELDF, C.S + EF0 + ESF + f * EF, r, cc, qc, rc);
+                E.L[f] = s_add(s_fma(T(-30), s_sub(cc, cm), qm), rc);
+                E.q[f] = qc;
+                E.c[f] = cc;
+            }
+        }
+        // planes 0 and 1 have fewer cubes to add; the rest is one straight body
+        Slots Z{1, 2, 0, 0, RP - 1, 0};
+        plane<ROLE, 0>(C, A, Z, Q, H, E, 0);
+        plane<ROLE, 1>(C, A, Z, Q, H, E, 1);
+        // (unrolled by two: 120 us against 117 at 256^3, spills in the step warps)
+#pragma unroll 1
+        for (int k = 2; k <= C.nz; k++) plane<ROLE, 2>(C, A, Z, Q, H, E, k);
+        __syncthreads();
+        if constexpr (ROLE == kSum)
+            cubes<true>(C, A, H, C.S + G0 + (Z.g ^ 1) * SLOTP, C.S + EG0 + (Z.g ^ 1) * ESP);
+    }
+
+    // The runs of the block's group, for a warp of pair row `row` (look-ahead warp:
+    // 0) of its tiles.
+    template <int ROLE>
+    static __device__ __forceinline__ void walk(Ctx& C, Acc& A, TileWalk runs, int nyt, int x0, int row)
+    {
+        const int n = C.n;
+        int yt;
+        for (bool first = true; runs.run(yt, C.z0, C.nz); first = false) {
+            runs.took(C.nz);
+            const int y0 = 2 * (yt * (n / 2) / nyt);
+            C.ty = 2 * ((yt + 1) * (n / 2) / nyt) - y0;
+            C.row = ROLE == kAhead ? C.ty + 1 : row;
+            C.offF = (uint32_t)C.row * RS + C.lane * VW;
+            C.offP = (uint32_t)(C.row - 1) * W + C.lane * VW;
+            const uint32_t xg = x0 + C.lane * VW;
+            C.rowg = (uint32_t)wrapn(y0 + C.row - 1, n) * n + xg;
+            C.rowlo = (uint32_t)wrapn(y0 - 1, n) * n + xg;
+            C.rowhi = (uint32_t)wrapn(y0 + C.ty + 1, n) * n + xg;
+            C.ey = (uint32_t)wrapn(y0 - 1 + min(C.lane, C.ty + 2), n) * n;
+            C.eyp = (uint32_t)wrapn(y0 + min(C.lane, C.ty), n) * n;
+            // every thread is done with the previous segment's ring before the
+            // prologue refills it
+            if (!first) __syncthreads();
+            if (ROLE == kAhead || row <= C.ty) run<ROLE>(C, A);
+            else run<kIdle>(C, A);
+        }
     }
 };
 
-template <typename T, int N, int TY, int D>
-__global__ void __launch_bounds__(S27<T, N, TY, D>::THREADS, 1)
+template <typename T, int TY, int D, bool EDGE>
+__global__ void __launch_bounds__(S27<T, TY, D, EDGE>::THREADS, 1)
     step27w_kernel(Bufs<T> B, Model M, DevScalars* sc, double* partials)
 {
-    typedef S27<T, N, TY, D> F;
-    constexpr int VW = F::VW, W = F::W, NXT = F::NXT;
+    typedef S27<T, TY, D, EDGE> F;
+    constexpr int VW = F::VW;
     __shared__ double red[32 * kSums];
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    chain_begin();
-    if (sc->status != LAT_OK) return;
 
     typename F::Ctx C;
     C.S = reinterpret_cast<T*>(smem_raw);
-    C.rho = threadIdx.x >> 5;                      // the warp's staged row, or ROWS for the edge warp
+    const int warp = threadIdx.x >> 5;
+    // warps: a step warp for each pair, then the look-ahead warp, then a
+    // sum warp for each pair
     C.lane = threadIdx.x & 31;
-    C.offF = (uint32_t)C.rho * F::RS + C.lane * VW;
-    C.offP = (uint32_t)(C.rho >= 1 && C.rho <= F::GR ? C.rho - 1 : 0) * W + C.lane * VW;
+    // groups of nxt blocks: the x tiles of one y tile, marching the same (y tile, z
+    // plane) units (lat_layout.cuh); the row's vectors are shared
+    // evenly among the x tiles, cut at multiples of 64 bytes where the row is one,
+    // the pairs of rows among the y tiles
+    const int n = M.n;
+    C.n = n;
+    C.nn = (uint32_t)n * n;
+    const int Q = n / VW, cut = Q % 4 == 0 ? 4 : Q % 2 == 0 ? 2 : 1;
+    const int nxt = EDGE ? (Q + 31) / 32 : 1, nyt = (n + TY - 1) / TY;
+    const int ngroups = gridDim.x / nxt;
+    const int grp = blockIdx.x / nxt, xt = blockIdx.x - grp * nxt;
+    const int q0 = xt * (Q / cut) / nxt * cut, qn = (xt + 1) * (Q / cut) / nxt * cut - q0;
+    const int x0 = q0 * VW, x1 = x0 + qn * VW;
+    C.last = qn - 1;
+    C.act = C.lane < qn;
+    // EDGE: what the end lanes get from the shuffles is replaced by edge scalars
+    C.sl = EDGE ? max(C.lane - 1, 0) : C.lane == 0 ? C.last : C.lane - 1;
+    C.sr = EDGE ? min(C.lane + 1, 31) : C.lane >= C.last ? 0 : C.lane + 1;
+    C.exl = (uint32_t)(x0 == 0 ? n - 1 : x0 - 1);
+    C.exr = (uint32_t)(x1 == n ? 0 : x1);
+    C.exr1 = (uint32_t)(x1 + 1 >= n ? x1 + 1 - n : x1 + 1);
+    TileWalk runs(nyt, ngroups, grp, n);
+
+    chain_begin();
+    if (sc->status != LAT_OK) return;
     const bool par = (sc->step & 1) != 0;
     C.f0 = par ? B.f[1][0] : B.f[0][0];
     C.f1 = par ? B.f[1][1] : B.f[0][1];
@@ -495,76 +661,47 @@ __global__ void __launch_bounds__(S27<T, N, TY, D>::THREADS, 1)
     C.op0 = par ? B.p[0][0] : B.p[1][0];
     C.op1 = par ? B.p[0][1] : B.p[1][1];
     C.K = site_coefs<T>(sc, M.beta);
-    const typename F::P zero = mk2(T(0), T(0));
-    C.wg[0] = C.wg[1] = C.vd = C.vi = zero;
-
-    // groups of NXT blocks: the x tiles of one y tile, marching the same
-    // (y tile, z plane) units (an equal share of the (N / TY) * N units per group)
-    const int ngroups = gridDim.x / NXT;
-    const int grp = blockIdx.x / NXT, xt = blockIdx.x - grp * NXT;
-    const int x0 = xt * W;
-    C.exl = (uint32_t)(x0 == 0 ? N - 1 : x0 - 1);
-    C.exr = (uint32_t)(x0 + W == N ? 0 : x0 + W);
-    C.exr1 = (uint32_t)(x0 + W + 1 >= N ? x0 + W + 1 - N : x0 + W + 1);
-    constexpr long long U = (long long)(N / TY) * N;
-    long long u = (long long)grp * U / ngroups;
-    const long long uend = ((long long)grp + 1) * U / ngroups;
-    for (bool first = true; u < uend; first = false) {
-        const int yt = (int)(u / N);
-        C.z0 = (int)(u - (long long)yt * N);
-        C.nz = (int)min((long long)(N - C.z0), uend - u);
-        u += C.nz;
-        C.rowg = (uint32_t)wrapn(yt * TY - 1 + (F::edge_warp(C) ? 0 : C.rho), N) * N + x0 + C.lane * VW;
-        C.ey = (uint32_t)wrapn(yt * TY - 1 + min(C.lane, F::ROWS - 1), N) * N;
-        C.eyp = (uint32_t)wrapn(yt * TY + min(C.lane, F::GR - 1), N) * N;
-        // every thread is done with the previous segment's ring before the
-        // prologue refills it
-        if (!first) __syncthreads();
-        // the same barriers on every path: one per plane, one after the run
-        if (F::edge_warp(C)) F::template run<kEdge>(C);
-        else if (C.rho == 0 || C.rho == F::ROWS - 1) F::template run<kStage>(C);
-        else if (C.rho == F::GR) F::template run<kAhead>(C);
-        else F::template run<kOwn>(C);
-        // the last bonds: planes nz - 1 and nz (the look-ahead plane)
-        __syncthreads();
-        if (!F::edge_warp(C) && C.rho >= 1 && C.rho <= TY) {
-            const int gb = (C.nz - 1) % F::GS, gl = C.nz % F::GS;
-            F::bonds(C, C.S + F::G0 + gb * F::SLOTP, C.S + F::G0 + gl * F::SLOTP, C.S + F::EG0 + gb * F::ESP,
-                     C.S + F::EG0 + gl * F::ESP);
-        }
+    typename F::Acc A;
+    A.wg[0] = A.wg[1] = A.vd = A.vi = mk2(T(0), T(0));
+    if (warp < F::PAIRS) F::template walk<kStep>(C, A, runs, nyt, x0, 2 * warp + 1);
+    else if (warp == F::PAIRS) F::template walk<kAhead>(C, A, runs, nyt, x0, 0);
+    else {
+        typename F::Acc S = A;
+        F::template walk<kSum>(C, S, runs, nyt, x0, 2 * (warp - F::PAIRS) - 1);
+        if (C.act) A = S;   // nothing in the other lanes
     }
 
-    double v[kSums];
-    for (int f = 0; f < 2; f++) v[f] = (double)lo2(C.wg[f]) + (double)hi2(C.wg[f]);
-    v[2] = ((double)lo2(C.vd) + (double)hi2(C.vd)) * (double)site_vsum_factor<T>(C.K.quartic);
-    v[3] = 0.5 * ((double)lo2(C.vi) + (double)hi2(C.vi));
-    finish_block(M, sc, partials, v, red, true);
+    // the pairs' two halves are added with their rounding errors beside them
+    TreeSum<T> v[kSums];
+    const T vf = site_vsum_factor<T>(C.K.quartic);   // factors of 1/2 and 1/4 are exact
+    auto both = [](typename F::P p, T f) {
+        TreeSum<T> a, b;
+        a.init(f * lo2(p));
+        b.init(f * hi2(p));
+        a.add(b);
+        return a;
+    };
+    v[0] = both(A.wg[0], T(1));
+    v[1] = both(A.wg[1], T(1));
+    v[2] = both(A.vd, vf);
+    v[3] = both(A.vi, T(0.5));
+    finish_block_trees<T>(M, sc, partials, v, red, true);
 }
 
-// Compiled instances: (element bytes, N, TY, D).
-struct Key27W {
-    int esize, n, ty, depth;
-};
-constexpr Key27W k27W[] = {{4, 256, 16, 1}, {4, 512, 16, 1}, {8, 256, 16, 1}, {8, 512, 16, 1}};
-
+// The compiled instance for a side, tile height and prefetch depth, or null.
 template <typename T>
 const void* s27w_fn(int n, int ty, int depth, size_t* smem)
 {
-#define LAT_S27W_CASE(NN, TT, DD)                                \
-    if (n == NN && ty == TT && depth == DD) {                    \
-        *smem = S27<T, NN, TT, DD>::SMEM;                        \
-        return (const void*)step27w_kernel<T, NN, TT, DD>;       \
+    constexpr bool kRows = sizeof(T) == 4;   // sides up to 64 are the plane-ring kernel's: FP64 rows are always cut
+    const bool edge = n > 32 * (int)(16 / sizeof(T));
+#define LAT_S27W_CASE(TT, DD)                                                  \
+    if (ty == TT && depth == DD) {                                             \
+        *smem = edge ? S27<T, TT, DD, true>::SMEM : S27<T, TT, DD, !kRows>::SMEM; \
+        return edge ? (const void*)step27w_kernel<T, TT, DD, true>             \
+                    : (const void*)step27w_kernel<T, TT, DD, !kRows>;          \
     }
-    LAT_S27W_CASE(256, 16, 1) LAT_S27W_CASE(512, 16, 1)
+    LAT_S27W_CASE(14, 2) LAT_S27W_CASE(16, 1)
 #undef LAT_S27W_CASE
-    return nullptr;
-}
-
-const void* s27w_kernel(int esize, int n, int ty, int depth, size_t* smem)
-{
-    for (const Key27W& k : k27W)
-        if (k.esize == esize && k.n == n && k.ty == ty && k.depth == depth)
-            return esize == 4 ? s27w_fn<float>(n, ty, depth, smem) : s27w_fn<double>(n, ty, depth, smem);
     return nullptr;
 }
 
@@ -572,20 +709,29 @@ const void* s27w_kernel(int esize, int n, int ty, int depth, size_t* smem)
 
 bool s27w_config(int n, int elem_bytes, int ty, int zr, int depth, MarchConfig* cfg)
 {
-    const int tyv = ty > 0 ? ty : 16;
-    const int d = depth > 0 ? depth : 1;
+    // FP32: tiles of 14 rows, two planes in flight (15 warps, 128 registers each,
+    // nothing spilled): 256^3 118 us per step against 129 with 16 rows (17 warps, 96
+    // registers), 512^3 823 against 911, 100^3 19.1 against 19.4; one plane in flight
+    // 124 and 877. FP64 is bound by its FP64 pipe, so the rows computed count: 16
+    // where they divide a larger side (128^3 499 against 541 us, 160^3 1070 against
+    // 1118, 256^3 3512 against 3570), else 14 (96^3 289 against 302, 132^3 790
+    // against 831).
+    const int best = elem_bytes == 8 && n % 16 == 0 && n >= 128 ? 16 : 14;
+    const int tyv = ty > 0 ? ty : depth > 0 ? (depth == 1 ? 16 : 14) : best;
+    const int d = depth > 0 ? depth : tyv == 14 ? 2 : 1;
     size_t smem = 0;
-    const void* fn = s27w_kernel(elem_bytes, n, tyv, d, &smem);
-    if (!fn || smem > 227 * 1024 - 2048) return false;
-    const int vw = 16 / elem_bytes, w = 32 * vw, nxt = n / w;
-    const int threads = (tyv + 4) * 32;
+    const void* fn = elem_bytes == 4 ? s27w_fn<float>(n, tyv, d, &smem) : s27w_fn<double>(n, tyv, d, &smem);
+    // up to 64 the plane-ring kernel (variant 2) runs every side
+    if (!fn || smem > 227 * 1024 - 2048 || n <= 64) return false;
+    const int vw = 16 / elem_bytes, nxt = (n / vw + 31) / 32;
+    const int threads = (tyv + 1) * 32;
     if (allow_dynamic_smem(fn, smem) != cudaSuccess) return false;
     int occ = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, threads, smem) != cudaSuccess || occ < 1) return false;
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) return false;
-    const int nyt = n / tyv;
+    const int nyt = (n + tyv - 1) / tyv;
     const long long tiles = (long long)nyt * nxt, units = tiles * n;
     long long blocks = 0;
     // whole groups of nxt blocks (the x tiles of a y tile, marching together)
@@ -594,7 +740,8 @@ bool s27w_config(int n, int elem_bytes, int ty, int zr, int depth, MarchConfig* 
     if (blocks < nxt) return false;
     const long long groups = blocks / nxt;
     cfg->ty = tyv;
-    cfg->zr = (int)(((long long)nyt * n + groups - 1) / groups);
+    const Layout L0 = tile_layout(nyt, (int)groups, 0, n);   // the first group's first run
+    cfg->zr = std::min(L0.uend - L0.ubeg, L0.zspan);
     cfg->nzc = (int)((groups + nyt - 1) / nyt);
     cfg->depth = d;
     cfg->threads = threads;
