@@ -139,11 +139,11 @@ size_t partials_needed(int n)
 
 // The L = 1/H form (expansion 2) solves the next step's coefficients in a pass
 // of its own after the sums (and after every step).
-lat_status launch_lform_pass(lat_handle* h)
+lat_status launch_lform_pass(lat_handle* h, bool chain)
 {
     if (h->M.expansion != 2) return LAT_OK;
-    cudaError_t e = h->prec == 32 ? launch_lform<float>(bufs_of<float>(h), h->M, h->sc, h->partials, h->stream)
-                                  : launch_lform<double>(bufs_of<double>(h), h->M, h->sc, h->partials, h->stream);
+    cudaError_t e = h->prec == 32 ? launch_lform<float>(bufs_of<float>(h), h->M, h->sc, h->partials, chain, h->stream)
+                                  : launch_lform<double>(bufs_of<double>(h), h->M, h->sc, h->partials, chain, h->stream);
     return cuda_status(e);
 }
 
@@ -152,7 +152,7 @@ lat_status launch_prepare(lat_handle* h)
     cudaError_t e = h->prec == 32 ? launch_sums<float>(bufs_of<float>(h), h->M, h->sc, h->partials, h->stream)
                                   : launch_sums<double>(bufs_of<double>(h), h->M, h->sc, h->partials, h->stream);
     LAT_TRY(cuda_status(e));
-    return launch_lform_pass(h);
+    return launch_lform_pass(h, false);
 }
 
 // One step of the configured kernel on the given buffers (the handle's own for
@@ -162,9 +162,10 @@ template <typename T>
 cudaError_t launch_step_with(lat_handle* h, const Bufs<T>& b, bool chain)
 {
     MarchConfig cfg = h->mcfg;
-    // not behind the L = 1/H form's pass: its blocks, set up beside the step's, keep
-    // the step's shared-memory split of L1 (256^3: 202 us per step chained, 198 not)
-    cfg.chain = chain && h->M.expansion != 2;
+    // not around the L = 1/H form's FP64 pass: its blocks, set up beside the step's,
+    // keep the step's shared-memory split of L1 (the FP32 pass in that form, 256^3:
+    // 202 us per step chained, 198 not)
+    cfg.chain = chain && (h->M.expansion != 2 || h->esize == 4);
     return launch_step_march<T>(b, h->M, h->sc, h->partials, cfg, h->stream);
 }
 template cudaError_t launch_step_with<float>(lat_handle*, const Bufs<float>&, bool);
@@ -175,7 +176,7 @@ lat_status launch_one_step(lat_handle* h, bool chain)
     cudaError_t e = h->prec == 32 ? launch_step_with<float>(h, bufs_of<float>(h), chain)
                                   : launch_step_with<double>(h, bufs_of<double>(h), chain);
     LAT_TRY(cuda_status(e));
-    return launch_lform_pass(h);
+    return launch_lform_pass(h, true);
 }
 
 void drop_graph(lat_handle* h)

@@ -163,7 +163,11 @@ cudaError_t launch_energy_field(const Bufs<T>& b, const Model& M, const DevScala
 // The L = 1/H form (expansion 2): the read-only pass over the current state
 // whose last block solves the next step's coefficients (lat_lform.cu).
 template <typename T>
-cudaError_t launch_lform(const Bufs<T>& b, const Model& M, DevScalars* sc, double* partials, cudaStream_t st);
+cudaError_t launch_lform(const Bufs<T>& b, const Model& M, DevScalars* sc, double* partials, bool chain, cudaStream_t st);
+// The FP32 form, over the step kernels' plane ring (lat_lform_ring.cu); `chain` as in
+// MarchConfig (FP64: never chained).
+cudaError_t launch_lform_ring(const Bufs<float>& b, const Model& M, DevScalars* sc, double* partials, bool chain,
+                              cudaStream_t st);
 // Shell sums of a half spectrum: out (3 nbins doubles) = [sum of |F|^2 / N^3, sum of
 // 2 pi |n| / L, modes] per shell; scratch holds spectrum_scratch(n, nbins) doubles.
 size_t spectrum_scratch(int n, int nbins);

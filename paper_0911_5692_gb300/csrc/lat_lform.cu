@@ -232,11 +232,10 @@ __device__ inline SiteCoef<T> block_coefs(const Model& M, const DevScalars* sc, 
 // 7-point pass: one 16-byte vector (V sites along x) per thread and plane,
 // marching a z run with the vectors of the planes below and above in
 // registers; the y neighbours as vectors, the x neighbours beyond the vector as
-// two scalars. Items: (n/V vectors x n rows) columns cut into nzc z runs.
-// FP32: at most 128 registers, for 2 blocks (16 warps) per SM, each with the
-// loads of two planes in flight.
+// two scalars. Items: (n/V vectors x n rows) columns cut into nzc z runs. (FP64; the
+// FP32 pass runs over the plane ring, lat_lform_ring.cu.)
 template <typename T>
-__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 2 : 1)
+__global__ void __launch_bounds__(256, 1)
     lform7_kernel(Bufs<T> B, Model M, DevScalars* sc, double* partials, int nzc)
 {
     constexpr int V = 16 / sizeof(T);
@@ -382,30 +381,34 @@ __global__ void __launch_bounds__(256) lform27_kernel(Bufs<T> B, Model M, DevSca
 } // namespace
 
 template <typename T>
-cudaError_t launch_lform(const Bufs<T>& b, const Model& M, DevScalars* sc, double* partials, cudaStream_t st)
+cudaError_t launch_lform(const Bufs<T>& b, const Model& M, DevScalars* sc, double* partials, bool chain, cudaStream_t st)
 {
-    const int n = M.n;
-    if (M.stencil == 27) {
-        lform27_kernel<T><<<sums_grid_blocks(n), 256, 0, st>>>(b, M, sc, partials, sums_zruns(n));
+    if constexpr (sizeof(T) == 4) {
+        return launch_lform_ring(b, M, sc, partials, chain, st);
+    } else {
+        const int n = M.n;
+        if (M.stencil == 27) {
+            lform27_kernel<T><<<sums_grid_blocks(n), 256, 0, st>>>(b, M, sc, partials, sums_zruns(n));
+            return cudaGetLastError();
+        }
+        // One resident wave of blocks (no more than the sums pass, whose partials
+        // buffer this pass shares); each thread marches whole z runs, two planes
+        // loaded before a run's first.
+        static int occ = 0;
+        const int wave = resident_wave((const void*)lform7_kernel<T>, 256, &occ);
+        if (wave == 0) return cudaErrorInvalidDevice;
+        constexpr int V = 16 / sizeof(T);
+        const long long vcols = (long long)(n / V) * n;
+        const int blocks_max = std::max(1, std::min(sums_grid_blocks(n), wave));
+        const int nzc = balanced_zruns(vcols, n, (long long)blocks_max * 256, 2.0);
+        const long long items = vcols * nzc;
+        const int blocks = (int)std::min<long long>(blocks_max, (items + 255) / 256);
+        lform7_kernel<T><<<blocks, 256, 0, st>>>(b, M, sc, partials, nzc);
         return cudaGetLastError();
     }
-    // One resident wave of blocks (no more than the sums pass, whose partials
-    // buffer this pass shares); each thread marches whole z runs, two planes
-    // loaded before a run's first.
-    static int occ = 0;
-    const int wave = resident_wave((const void*)lform7_kernel<T>, 256, &occ);
-    if (wave == 0) return cudaErrorInvalidDevice;
-    constexpr int V = 16 / sizeof(T);
-    const long long vcols = (long long)(n / V) * n;
-    const int blocks_max = std::max(1, std::min(sums_grid_blocks(n), wave));
-    const int nzc = balanced_zruns(vcols, n, (long long)blocks_max * 256, 2.0);
-    const long long items = vcols * nzc;
-    const int blocks = (int)std::min<long long>(blocks_max, (items + 255) / 256);
-    lform7_kernel<T><<<blocks, 256, 0, st>>>(b, M, sc, partials, nzc);
-    return cudaGetLastError();
 }
 
-template cudaError_t launch_lform<float>(const Bufs<float>&, const Model&, DevScalars*, double*, cudaStream_t);
-template cudaError_t launch_lform<double>(const Bufs<double>&, const Model&, DevScalars*, double*, cudaStream_t);
+template cudaError_t launch_lform<float>(const Bufs<float>&, const Model&, DevScalars*, double*, bool, cudaStream_t);
+template cudaError_t launch_lform<double>(const Bufs<double>&, const Model&, DevScalars*, double*, bool, cudaStream_t);
 
 } // namespace lat

@@ -61,6 +61,7 @@
 // and P + 1 is summed at plane P + 2, after the barrier that completes P + 1.
 #include <algorithm>
 
+#include "lat_agg27.cuh"
 #include "lat_async.cuh"
 #include "lat_kernels.h"
 #include "lat_layout.cuh"
@@ -215,74 +216,13 @@ struct S27 {
         }
     }
 
-    // The aggregates of one field at this lane's sites of its R rows: centres c,
-    // q = 3 e + k and r = 14 e + 3 k. F: the field's plane in the ring, E: its
-    // edge scalars. Every lane calls this.
+    // The aggregates of one field at this lane's sites of its R rows (lat_agg27.cuh).
+    // F: the field's plane in the ring, E: its edge scalars.
     template <int R>
     static __device__ __forceinline__ void aggr(const Ctx& C, const T* F, const T* E, P (&c)[R][NP], P (&q)[R][NP],
                                                 P (&r)[R][NP])
     {
-        const T* row = F + C.offF;
-        P up[NP], dn[NP], v[R][NP];
-        PK<T>::ld(row - RS, up);
-#pragma unroll
-        for (int i = 0; i < R; i++) PK<T>::ld(row + i * RS, c[i]);
-        PK<T>::ld(row + R * RS, dn);
-        // the column beside the tile's end that this lane is at, rows row - 1 ..
-        // row + R, and its y pairs
-        T ec[R + 2], ev[R];
-        const bool first = C.lane == 0, last = C.lane == C.last;
-        if constexpr (EDGE) {
-            const T* e = E + (C.row - 1) * 4 + (first ? 0 : 1);
-#pragma unroll
-            for (int i = 0; i < R + 2; i++) ec[i] = ld_shared_if(first || last, e + 4 * i, T(0));
-#pragma unroll
-            for (int i = 0; i < R; i++) ev[i] = s_add(s_sub(ec[i], ec[i + 1]), s_sub(ec[i + 2], ec[i + 1]));
-        }
-        // the y difference inside a pair serves both rows
-#pragma unroll
-        for (int j = 0; j < NP; j++) {
-            if constexpr (R == 2) {
-                const P in = sub2(c[1][j], c[0][j]);
-                v[0][j] = add2(sub2(up[j], c[0][j]), in);
-                v[1][j] = sub2(sub2(dn[j], c[1][j]), in);
-            } else {
-                v[0][j] = add2(sub2(up[j], c[0][j]), sub2(dn[j], c[0][j]));
-            }
-        }
-        const P two = mk2(T(2), T(2)), three = mk2(T(3), T(3)), fourteen = mk2(T(14), T(14));
-#pragma unroll
-        for (int i = 0; i < R; i++) {
-            T cs[VW + 2], vs[VW + 2];
-#pragma unroll
-            for (int j = 0; j < NP; j++) {
-                un2(c[i][j], cs[1 + 2 * j], cs[2 + 2 * j]);
-                un2(v[i][j], vs[1 + 2 * j], vs[2 + 2 * j]);
-            }
-            cs[0] = __shfl_sync(kFull, cs[VW], C.sl);
-            cs[VW + 1] = __shfl_sync(kFull, cs[1], C.sr);
-            vs[0] = __shfl_sync(kFull, vs[VW], C.sl);
-            vs[VW + 1] = __shfl_sync(kFull, vs[1], C.sr);
-            if constexpr (EDGE) {
-                cs[0] = first ? ec[i + 1] : cs[0];
-                vs[0] = first ? ev[i] : vs[0];
-                cs[VW + 1] = last ? ec[i + 1] : cs[VW + 1];
-                vs[VW + 1] = last ? ev[i] : vs[VW + 1];
-            }
-            T dd[VW + 1];   // differences of consecutive sites
-#pragma unroll
-            for (int x = 0; x <= VW; x++) dd[x] = s_sub(cs[x + 1], cs[x]);
-#pragma unroll
-            for (int j = 0; j < NP; j++) {
-                const int a = 1 + 2 * j, b = 2 + 2 * j;   // positions of the pair's sites in cs and vs
-                const P h = mk2(s_sub(dd[a], dd[a - 1]), s_sub(dd[b], dd[b - 1]));
-                const P t = mk2(s_add(vs[a - 1], vs[a + 1]), s_add(vs[b - 1], vs[b + 1]));
-                const P k = fma2(two, h, t);
-                const P eh = add2(h, v[i][j]);
-                q[i][j] = fma2(three, eh, k);
-                r[i][j] = fma2(fourteen, eh, mul2(three, k));
-            }
-        }
+        agg27<T, R, EDGE>(F + C.offF, RS, C.lane, C.last, C.sl, C.sr, E + (C.row - 1) * 4, 4, c, q, r);
     }
 
     // The same aggregates at one site, rounded as the first site of a vector:
