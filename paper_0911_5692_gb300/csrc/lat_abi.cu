@@ -257,16 +257,18 @@ lat_status configure_kernel(lat_handle* h, int variant, int ty, int zr, int dept
         // 2, 56^3: 10.8 against 12.9, 100^3: 15.7 against 19.8); rows cut into x tiles
         // from 21 lanes a tile on (160^3, 20 lanes: 42.1 against 41.8; 168^3, 21
         // lanes: 45.2 against 46.5; 384^3, 32 lanes: 298 against 435). Tiles of 16
-        // rows with two planes in flight where the lanes are full or the row is one
-        // tile (512^3: 685 us, 8 rows 718), else 8 rows with three, two blocks to an
-        // SM: with empty lanes a block moves fewer bytes per barrier (200^3: 62
-        // against 64 us, 464^3: 579 against 592, 496^3: 700 against 710, 704^3: 2050
-        // against 2138).
+        // rows with two planes in flight where the lanes are full (512^3: 685 us, 8
+        // rows 718) or a row of one tile is short (84^3: 13.4 against 13.7, 100^3 the
+        // same); of 8 rows for longer rows of one tile, where a group has planes enough
+        // for twice the tiles (108^3: 16.7 against 17.3, 116^3: 17.3 against 19.1,
+        // 128^3: 19.4 against 19.9); else 8 rows with three, two blocks to an SM: with
+        // empty lanes a block moves fewer bytes per barrier (200^3: 62 against 64 us,
+        // 464^3: 579 against 592, 496^3: 700 against 710, 704^3: 2050 against 2138).
         const int q = n / 4, nxt = (q + 31) / 32;
         MarchConfig cfg;
         if (nxt == 1 ? n >= 56 : q / nxt >= 21) {
-            const bool tall = nxt == 1 || q == 32 * nxt;
-            if (xw_config(n, 4, tall ? 16 : 8, 0, tall ? 2 : 3, &cfg) && fits(cfg)) return take(cfg, 5);
+            const bool tall = nxt == 1 ? n <= 100 : q == 32 * nxt;
+            if (xw_config(n, 4, tall ? 16 : 8, 0, tall || nxt == 1 ? 2 : 3, &cfg) && fits(cfg)) return take(cfg, 5);
         }
     }
     if (variant == 0 && n / (16 / (int)h->esize) >= 128) {

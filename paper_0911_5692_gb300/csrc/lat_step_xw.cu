@@ -10,8 +10,8 @@ namespace lat {
 namespace {
 
 // The compiled instance for a side, tile height and prefetch depth. FP32 sides of
-// at most 128 take whole rows in 16-row tiles with two planes in flight: without
-// the edge warp, and with two pairs of rows to a warp up to N = 64, a step is
+// at most 128 take whole rows in tiles of 16 or 8 rows with two planes in flight:
+// without the edge warp, and with two pairs of rows to a warp up to N = 64, a step is
 // 1.1 us (100^3: 16.8 -> 15.7) to 1.6 us (64^3: 12.6 -> 11.0) shorter.
 struct XWInst {
     const void* fn = nullptr;
@@ -29,6 +29,7 @@ XWInst xw_inst(int n, int ty, int depth)
     if constexpr (sizeof(T) == 4) {
         if (ty == 16 && depth == 2 && n <= 64) LAT_XW_CASE(16, 2, 16)
         if (ty == 16 && depth == 2 && n <= 128) LAT_XW_CASE(16, 2, 32)
+        if (ty == 8 && depth == 2 && n <= 128) LAT_XW_CASE(8, 2, 32)
         if (ty == 16 && depth == 3) LAT_XW_CASE(16, 3, 0)
         if (ty == 8 && depth == 2) LAT_XW_CASE(8, 2, 0)
         if (ty == 8 && depth == 3) LAT_XW_CASE(8, 3, 0)
