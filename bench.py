@@ -102,7 +102,7 @@ STEP_KERNEL_SOURCES = {
 
 
 VARIANT_SOURCES = {(7, 4): ("lat_step_xt.cu",), (7, 5): ("lat_step_xw.cu", "lat_xw.cuh", "lat_layout.cuh"),
-                   (27, 5): ("lat_step27w.cu",)}
+                   (27, 5): ("lat_step27w.cu", "lat_agg27.cuh", "lat_layout.cuh")}
 
 
 def kernel_source_hash(stencil=7, variant=2):

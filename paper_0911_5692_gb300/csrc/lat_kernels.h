@@ -80,8 +80,8 @@ bool xt_config(int n, int elem_bytes, int ty, int zr, int depth, MarchConfig* cf
 template <typename T>
 cudaError_t launch_step_xt(const Bufs<T>& b, const Model& M, DevScalars* sc, double* partials, const MarchConfig& cfg,
                            cudaStream_t st);
-// x tiles one warp wide with compile-time N, ty, depth and an edge warp for the
-// tile's x neighbours (whole periodic lattices; the compiled geometries only)
+// x tiles one warp wide, compiled for each ty and depth (lat_xw.cuh; whole periodic
+// lattices)
 bool xw_config(int n, int elem_bytes, int ty, int zr, int depth, MarchConfig* cfg);
 template <typename T>
 cudaError_t launch_step_xw(const Bufs<T>& b, const Model& M, DevScalars* sc, double* partials, const MarchConfig& cfg,
@@ -117,8 +117,7 @@ bool slab_xw_config(int n, int elem_bytes, int nz, MarchConfig* cfg);
 template <typename T>
 cudaError_t launch_slab_xw(const xw::SlabRun& R, const Model& M, DevScalars* sc, double* partials,
                            const MarchConfig& cfg, cudaStream_t st);
-// the 27-point Laplacian over x tiles one warp wide with compile-time N, ty,
-// depth and an edge warp (whole periodic lattices; the compiled geometries only)
+// the 27-point Laplacian over x tiles one warp wide (lat_step27w.cu; sides above 64)
 bool s27w_config(int n, int elem_bytes, int ty, int zr, int depth, MarchConfig* cfg);
 template <typename T>
 cudaError_t launch_step27w(const Bufs<T>& b, const Model& M, DevScalars* sc, double* partials, const MarchConfig& cfg,
