@@ -159,7 +159,7 @@ struct S27 {
     static __device__ __forceinline__ void fetch_f(const Ctx& C, int zrel, int slot)
     {
         const uint32_t zoff = (uint32_t)wrapn(C.z0 + zrel, C.n) * C.nn;
-        if constexpr (ROLE == kStep) {
+        if constexpr (ROLE == kSum) {
             const T *a = C.f0 + zoff + C.rowg, *b = C.f1 + zoff + C.rowg;
             T* d = C.S + slot * SLOTF + C.offF;
             if (C.act) {
@@ -196,13 +196,13 @@ struct S27 {
     static __device__ __forceinline__ void fetch_p(const Ctx& C, int zrel, int slot)
     {
         const uint32_t zoff = (uint32_t)wrapn(C.z0 + zrel, C.n) * C.nn;
-        if constexpr (ROLE == kStep || ROLE == kAhead) {
+        if constexpr (ROLE == kSum || ROLE == kAhead) {
             const T *a = C.p0 + zoff + C.rowg, *b = C.p1 + zoff + C.rowg;
             T* d = C.S + P0 + slot * SLOTP + C.offP;
             if (C.act) {
                 cp_async16(d, a);
                 cp_async16(d + FIELDP, b);
-                if constexpr (ROLE == kStep) {
+                if constexpr (ROLE == kSum) {
                     cp_async16(d + W, a + C.n);
                     cp_async16(d + FIELDP + W, b + C.n);
                 }
@@ -254,8 +254,8 @@ struct S27 {
     // from EG) and, where SUM is set, adds the cubes between plane P - 1 (in H) and
     // P, and the potential of plane P - 1; leaves plane P in H. Every lane calls
     // this.
-    template <bool SUM>
-    static __device__ __forceinline__ void cubes(const Ctx& C, Acc& A, Cube& H, const T* G, const T* EG)
+    template <bool SUM, bool STORE>
+    static __device__ __forceinline__ void cubes(const Ctx& C, Acc& A, Cube& H, const T* G, const T* EG, int k)
     {
         const bool last = C.lane == C.last;
         const T* gp = G + (C.row - 1) * W + C.lane * VW;
@@ -273,6 +273,11 @@ struct S27 {
             T re[3];
 #pragma unroll
             for (int i = 0; i < 3; i++) PK<T>::ld(gp + f * FIELDP + i * W, g[i]);
+            if (STORE && C.act) {
+                T* o = (f ? C.of1 : C.of0) + (uint32_t)wrapn(C.z0 + k, C.n) * C.nn + C.rowg;
+                PK<T>::st_stream(o, g[0]);
+                PK<T>::st_stream(o + C.n, g[1]);
+            }
 #pragma unroll
             for (int i = 0; i < 3; i++) {
                 re[i] = __shfl_sync(kFull, lo2(g[i][0]), C.sr);
@@ -426,8 +431,6 @@ struct S27 {
             for (int i = 0; i < R; i++) {
                 PK<T>::st_stream(C.op0 + gi + i * C.n, pn[0][i]);
                 PK<T>::st_stream(C.op1 + gi + i * C.n, pn[1][i]);
-                PK<T>::st_stream(C.of0 + gi + i * C.n, g[0][i]);
-                PK<T>::st_stream(C.of1 + gi + i * C.n, g[1][i]);
             }
         }
 #pragma unroll
@@ -443,13 +446,13 @@ struct S27 {
     {
         cp_async_wait(D - 1);
         __syncthreads();
-        if ((ROLE == kStep || ROLE == kAhead) && k + D <= C.nz) {
+        if ((ROLE == kSum || ROLE == kAhead) && k + D <= C.nz) {
             fetch_f<ROLE>(C, k + D + 1, Z.fw);
             fetch_p<ROLE>(C, k + D, Z.pw);
         }
         cp_async_commit();
         if constexpr (ROLE == kSum && BEHIND > 0)
-            cubes<(BEHIND > 1)>(C, A, H, C.S + G0 + (Z.g ^ 1) * SLOTP, C.S + EG0 + (Z.g ^ 1) * ESP);
+            cubes<(BEHIND > 1), true>(C, A, H, C.S + G0 + (Z.g ^ 1) * SLOTP, C.S + EG0 + (Z.g ^ 1) * ESP, k - 1);
         if constexpr (EDGE && ROLE == kAhead) plane_edge(C, Z, E);
         if constexpr (ROLE == kStep || ROLE == kAhead) plane_rows<R>(C, Z, Q, k);
         Z.next();
@@ -519,7 +522,7 @@ struct S27 {
         for (int k = 2; k <= C.nz; k++) plane<ROLE, 2>(C, A, Z, Q, H, E, k);
         __syncthreads();
         if constexpr (ROLE == kSum)
-            cubes<true>(C, A, H, C.S + G0 + (Z.g ^ 1) * SLOTP, C.S + EG0 + (Z.g ^ 1) * ESP);
+            cubes<true, false>(C, A, H, C.S + G0 + (Z.g ^ 1) * SLOTP, C.S + EG0 + (Z.g ^ 1) * ESP, C.nz);
     }
 
     // The runs of the block's group, for a warp of pair row `row` (look-ahead warp:
