@@ -6,23 +6,26 @@
 // Tiles, ring and layout follow the 7-point kernel of lat_xw.cuh: a tile is at most
 // W = 32 16-byte vectors wide (a row's vectors are shared evenly among its tiles)
 // and at most TY rows tall. Two warps serve each pair of neighbouring rows: the step
-// warp kicks and drifts it, the sum warp adds up the new fields one plane later.
+// warp kicks and drifts it and stores its momenta; the sum warp stages the pair's
+// rows, and one plane later adds up the new fields and stores them.
 // One more warp stages the halo rows, kicks and drifts the look-ahead row, and,
 // where the row is cut into x tiles, stages the scalars of the tile's x neighbours
 // (columns x0 - 1 and the two right of the tile) and computes the new fields of
 // the boundary column right of the tile, rounded exactly as the next tile computes
 // its own first column. Rows of one tile reach their ends by a rotating shuffle.
 //
-// What bounds it. FP32: the instructions of a plane, about 500 per row of a warp
-// (990 per pair against some 1500 with one row per warp and 13 squared bonds per
-// site), issued by 15 warps; the copy itself would take 79 us of the 117 at 256^3.
-// One warp for both halves of a pair's work held 252 registers, two warps to a
-// scheduler, and waited on its own latencies (issue slots 43 % busy, 126 us at
-// 256^3, 913 at 512^3); the two halves in two warps of 128 registers overlap, with
-// the new fields through shared memory: 117 and 824 us. One row per warp took 149
-// and 1187. Sides that only the plane-ring kernel ran before: 100^3 42 -> 19 us,
-// 292^3 1690 -> 206, 384^3 699 -> 369, 1024^3 13.4 -> 6.4 ms. FP64 is bound by the
-// FP64 pipe: 256^3 4.07 -> 3.51 ms.
+// What bounds it. FP32: the instructions of a plane, about 480 per row of a warp (960
+// per pair against some 1500 with one row per warp and 13 squared bonds per site),
+// issued by 15 warps, and the step warps' chain from barrier to barrier; the copy
+// itself would take 79 us of the 107 at 256^3 and 636 of the 760 at 512^3. One warp
+// for both halves of a pair's work held 252 registers, two warps to a scheduler,
+// and waited on its own latencies (issue slots 43 % busy, 126 us at 256^3, 913 at
+// 512^3); the two halves in two warps of 128 registers overlap, with the new fields
+// through shared memory (117 and 824 us), and with the copies and the fields'
+// stores on the sum warps, which waited for the others at the barrier, 107 and 760.
+// One row per warp took 149 and 1187. Sides that only the plane-ring kernel ran
+// before: 100^3 42 -> 18 us, 292^3 1690 -> 188, 384^3 699 -> 334. FP64 is bound by
+// the FP64 pipe: 256^3 4.07 -> 3.50 ms.
 //
 // Laplacian. In units of 1/(30 dx^2) the weights are 14 (6 faces), 3 (12 edges)
 // and 1 (8 corners). Per plane p and site, with differences taken from that
@@ -517,7 +520,7 @@ struct S27 {
         Slots Z{1, 2, 0, 0, RP - 1, 0};
         plane<ROLE, 0>(C, A, Z, Q, H, E, 0);
         plane<ROLE, 1>(C, A, Z, Q, H, E, 1);
-        // (unrolled by two: 120 us against 117 at 256^3, spills in the step warps)
+        // (unrolled by two it was 120 us against 117 at 256^3, with spills)
 #pragma unroll 1
         for (int k = 2; k <= C.nz; k++) plane<ROLE, 2>(C, A, Z, Q, H, E, k);
         __syncthreads();
@@ -653,11 +656,11 @@ const void* s27w_fn(int n, int ty, int depth, size_t* smem)
 bool s27w_config(int n, int elem_bytes, int ty, int zr, int depth, MarchConfig* cfg)
 {
     // FP32: tiles of 14 rows, two planes in flight (15 warps, 128 registers each,
-    // nothing spilled): 256^3 118 us per step against 129 with 16 rows (17 warps, 96
-    // registers), 512^3 823 against 911, 100^3 19.1 against 19.4; one plane in flight
-    // 124 and 877. FP64 is bound by its FP64 pipe, so the rows computed count: 16
-    // where they divide a larger side (128^3 499 against 541 us, 160^3 1070 against
-    // 1118, 256^3 3512 against 3570), else 14 (96^3 289 against 302, 132^3 790
+    // nothing spilled): 256^3 107 us per step against 151 with 16 rows and one plane
+    // (17 warps, 96 registers), 512^3 760 against 1108, 100^3 17.9 against 18.8; 14 rows
+    // with one plane in flight 120 and 879, with three 111 and 770. FP64 is bound by its FP64 pipe, so the rows computed count: 16
+    // where they divide a larger side (128^3 496 against 538 us, 160^3 1070 against
+    // 1118, 256^3 3497 against 3539), else 14 (96^3 289 against 302, 132^3 790
     // against 831).
     const int best = elem_bytes == 8 && n % 16 == 0 && n >= 128 ? 16 : 14;
     const int tyv = ty > 0 ? ty : depth > 0 ? (depth == 1 ? 16 : 14) : best;
