@@ -963,27 +963,44 @@ lat_status vjp_impl(lat_handle* h, int64_t n, int64_t ckpt_every, T* fb_user, T*
         }
         return b;
     };
-    for (int64_t k = 0; k < n; k++) {
-        const int par = (int)((s0.step + k) & 1);
-        if (k % K == 0) {
-            T* c = arr(ck, (size_t)(k / K) * 6);
-            for (int f = 0; f < 2; f++) {
-                LAT_CUDA(cudaMemcpyAsync(c + f * N3, hb.f[par][f], ab, cudaMemcpyDeviceToDevice, st));
-                LAT_CUDA(cudaMemcpyAsync(c + (2 + f) * N3, hb.p[par][f], ab, cudaMemcpyDeviceToDevice, st));
-                if (k > 0) LAT_CUDA(cudaMemcpyAsync(c + (4 + f) * N3, hb.f[1 - par][f], ab, cudaMemcpyDeviceToDevice, st));
+    auto forward = [&]() -> lat_status {
+        for (int64_t k = 0; k < n; k++) {
+            const int par = (int)((s0.step + k) & 1);
+            if (k % K == 0) {
+                T* c = arr(ck, (size_t)(k / K) * 6);
+                for (int f = 0; f < 2; f++) {
+                    LAT_CUDA(cudaMemcpyAsync(c + f * N3, hb.f[par][f], ab, cudaMemcpyDeviceToDevice, st));
+                    LAT_CUDA(cudaMemcpyAsync(c + (2 + f) * N3, hb.p[par][f], ab, cudaMemcpyDeviceToDevice, st));
+                    if (k > 0) LAT_CUDA(cudaMemcpyAsync(c + (4 + f) * N3, hb.f[1 - par][f], ab, cudaMemcpyDeviceToDevice, st));
+                }
+                LAT_CUDA(cudaMemcpyAsync(ck_sc + k / K, h->sc, sizeof(DevScalars), cudaMemcpyDeviceToDevice, st));
+                if (k == clast)
+                    for (int f = 0; f < 2; f++)
+                        LAT_CUDA(cudaMemcpyAsync(arr(seg, f), hb.f[par][f], ab, cudaMemcpyDeviceToDevice, st));
             }
-            LAT_CUDA(cudaMemcpyAsync(ck_sc + k / K, h->sc, sizeof(DevScalars), cudaMemcpyDeviceToDevice, st));
-            if (k == clast)
-                for (int f = 0; f < 2; f++)
-                    LAT_CUDA(cudaMemcpyAsync(arr(seg, f), hb.f[par][f], ab, cudaMemcpyDeviceToDevice, st));
+            LAT_CUDA(launch_step_with<T>(h, k < clast ? hb : seg_bufs(k, clast), k % K != 0));
         }
-        LAT_CUDA(launch_step_with<T>(h, k < clast ? hb : seg_bufs(k, clast), k % K != 0));
+        return LAT_OK;
+    };
+    rs = forward();
+    const lat_status cleared = guard.clear();
+    // The fields of the step reached go back into the handle's own set: f_n, or those of
+    // an earlier step when its sums were not finite (the steps after it return at once
+    // and leave their part of seg unwritten) or a launch was refused. Up to clast the
+    // handle's own arrays hold them. (Reading the scalars here costs nothing that shows:
+    // 128^3 FP32, 100 steps, 8.60 and 8.61 ms without and with.)
+    DevScalars s1;
+    LAT_TRY(read_scalars(h, &s1));
+    const int64_t past = s1.step - s0.step - clast;
+    for (int f = 0; f < 2 && past > 0; f++)
+        LAT_CUDA(cudaMemcpyAsync(hb.f[s1.step & 1][f], arr(seg, (size_t)past * 2 + f), ab, cudaMemcpyDeviceToDevice, st));
+    if (rs == LAT_OK) rs = cleared;
+    if (rs == LAT_OK) rs = (lat_status)s1.status;
+    if (rs != LAT_OK) {   // no observable, no reverse sweep: the scratch goes once the copy is done
+        LAT_CUDA(cudaStreamSynchronize(st));
+        return rs;
     }
-    LAT_TRY(guard.clear());
     const int parN = (int)((s0.step + n) & 1);
-    if (n > 0)   // f_n back into the handle's own set
-        for (int f = 0; f < 2; f++)
-            LAT_CUDA(cudaMemcpyAsync(hb.f[parN][f], arr(seg, (size_t)(n - clast) * 2 + f), ab, cudaMemcpyDeviceToDevice, st));
     for (int f = 0; f < 2; f++) {
         LAT_CUDA(cudaMemcpyAsync(fin + f * N3, hb.f[parN][f], ab, cudaMemcpyDeviceToDevice, st));
         LAT_CUDA(cudaMemcpyAsync(fin + (2 + f) * N3, hb.p[parN][f], ab, cudaMemcpyDeviceToDevice, st));
@@ -1124,10 +1141,7 @@ lat_status vjp_impl(lat_handle* h, int64_t n, int64_t ckpt_every, T* fb_user, T*
     LAT_CUDA(cudaMemcpyAsync(h->sc, fin_sc, sizeof(DevScalars), cudaMemcpyDeviceToDevice, st));
     AdjScalars out;
     LAT_CUDA(cudaMemcpyAsync(&out, as, sizeof(out), cudaMemcpyDeviceToHost, st));
-    DevScalars sN;
-    LAT_CUDA(cudaMemcpyAsync(&sN, fin_sc, sizeof(sN), cudaMemcpyDeviceToHost, st));
     LAT_CUDA(cudaStreamSynchronize(st));
-    if (sN.status != LAT_OK) return (lat_status)sN.status;
     if (out.status != LAT_OK) return (lat_status)out.status;
     sbar[0] = out.ba;
     sbar[1] = out.bad;
