@@ -25,19 +25,25 @@ __device__ __forceinline__ void cp_async_small(void* smem, const void* gmem)
                  "l"(gmem), "n"(BYTES)
                  : "memory");
 }
-// v, or the shared-memory value at a where p holds: a predicated load, no branch
+// v, or the shared-memory value at a where p holds: a predicated load, no branch.
+// Volatile with a memory clobber, as a plain load is to the compiler: two uses with
+// equal operands are two loads, and none moves across a store, a barrier or the wait
+// for a copy. (Registers, spills and times of every kernel as without; a plain load
+// under an if takes 244 -> 320 bytes of spills in the 27-point kernel of 16 rows.)
 __device__ __forceinline__ float ld_shared_if(bool p, const float* a, float v)
 {
-    asm("{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %2, 0;\n\t@q ld.shared.f32 %0, [%1];\n\t}"
+    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %2, 0;\n\t@q ld.shared.f32 %0, [%1];\n\t}"
         : "+f"(v)
-        : "r"((uint32_t)__cvta_generic_to_shared(a)), "r"((int)p));
+        : "r"((uint32_t)__cvta_generic_to_shared(a)), "r"((int)p)
+        : "memory");
     return v;
 }
 __device__ __forceinline__ double ld_shared_if(bool p, const double* a, double v)
 {
-    asm("{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %2, 0;\n\t@q ld.shared.f64 %0, [%1];\n\t}"
+    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %2, 0;\n\t@q ld.shared.f64 %0, [%1];\n\t}"
         : "+d"(v)
-        : "r"((uint32_t)__cvta_generic_to_shared(a)), "r"((int)p));
+        : "r"((uint32_t)__cvta_generic_to_shared(a)), "r"((int)p)
+        : "memory");
     return v;
 }
 
