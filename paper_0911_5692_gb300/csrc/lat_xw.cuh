@@ -110,6 +110,22 @@ struct XW {
         P dtcl2, dtcf2;
         SiteCoefs<T> K;
     };
+    // A lane of the pair warps or of the look-ahead warp in a tile of ty rows and qn
+    // vectors: its (first) row in the staged tile, whether it holds a vector of it (lx
+    // in its row), and where that lies in the new-field plane.
+    static __host__ __device__ __forceinline__ int pair_of(int warp, int lane) { return warp * RPW + lane / LW; }
+    static __host__ __device__ __forceinline__ int row_of(bool ahead, int pair, int ty) { return ahead ? ty + 1 : 2 * pair + 1; }
+    static __host__ __device__ __forceinline__ bool holds(bool ahead, int pair, int lane, int lx, int qn, int ty)
+    {
+        return EDGE ? lx < qn : lx < qn && (ahead ? lane < LW : 2 * pair < ty);
+    }
+    static __host__ __device__ __forceinline__ uint32_t off_g(int row, int lx) { return (uint32_t)((row - 1) / 2) * W + lx * VW; }
+    // Whether it stores its new field for the other warps. With several pairs to a warp
+    // the last warp may reach past the tile's last row, and a pair just past it lies
+    // where the look-ahead row does: the lanes that hold nothing store nothing, so that
+    // every vector of the plane has one writer. (With x tiles those lanes' vectors are
+    // their own.)
+    static __host__ __device__ __forceinline__ bool shares(bool act) { return EDGE || act; }
     // the ring slots of one plane step, as offsets: field plane k, k + 1 and the
     // slot that plane k - 1 left; momentum plane k and the slot that k - 1 left
     struct Slots {
@@ -338,8 +354,10 @@ struct XW {
                     PK<T>::st_stream(C.of1 + gi + r * C.n, g[1][r]);
                 }
             }
-            PK<T>::st(Gw, g[0][0]);
-            PK<T>::st(Gw + FIELDG, g[1][0]);
+            if (shares(C.act)) {
+                PK<T>::st(Gw, g[0][0]);
+                PK<T>::st(Gw + FIELDG, g[1][0]);
+            }
         }
         // sums over the owned rows of plane k-1 (x and y pairs, potential) and
         // the z pair (k-1, k); the row after the pair's second is the next pair's
@@ -478,16 +496,16 @@ struct XW {
         C.lx = C.lane % LW;
         C.ty = ty;
         C.last = qn - 1;
-        const int pair = warp * RPW + C.lane / LW;
-        C.act = EDGE ? C.lx < qn : C.lx < qn && (ahead ? C.lane < LW : 2 * pair < ty);
-        C.row = ahead ? ty + 1 : 2 * pair + 1;
+        const int pair = pair_of(warp, C.lane);
+        C.act = holds(ahead, pair, C.lane, C.lx, qn, ty);
+        C.row = row_of(ahead, pair, ty);
         if constexpr (!EDGE) {
             C.sl = C.lane - C.lx + (C.lx == 0 ? qn - 1 : C.lx - 1);
             C.sr = C.lane - C.lx + (C.lx + 1 >= qn ? 0 : C.lx + 1);
         }
         C.offF = (uint32_t)C.row * W + C.lx * VW;
         C.offP = (uint32_t)(C.row - 1) * W + C.lx * VW;
-        C.offG = (uint32_t)((C.row - 1) / 2) * W + C.lx * VW;
+        C.offG = off_g(C.row, C.lx);
         const int x0 = q0 * VW, x1 = x0 + qn * VW;
         const uint32_t xg = x0 + C.lx * VW;
         C.rowg = (uint32_t)wrapn(y0 + C.row - 1, n) * n + xg;
