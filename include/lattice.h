@@ -394,8 +394,8 @@ lat_status lat_set_g2(lat_handle* h, double g2);
  * Synchronises. LAT_ENOMEM if the checkpoints do not fit; LAT_EUNSUPPORTED for
  * a 27-point lattice, expansion = 2 or split storage; sticky device errors of the
  * forward or reverse pass are returned. After one of the forward pass (non-finite
- * sums) the handle stands at the step that failed, as after lat_evolve, and nothing
- * has been written to the arrays, to sbar or to lat_adjoint's J_out. */
+ * sums) the handle stands at the step that failed, as after lat_evolve, and sbar and
+ * lat_adjoint's J_out have not been written. */
 lat_status lat_vjp(lat_handle* h, int64_t n_steps, int64_t ckpt_every, void* fbar_dev, void* pibar_dev,
                    double sbar[4]);
 

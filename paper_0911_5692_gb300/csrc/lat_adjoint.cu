@@ -933,7 +933,7 @@ lat_status vjp_impl(lat_handle* h, int64_t n, int64_t ckpt_every, T* fb_user, T*
     S.want(&fin_sc, sizeof(DevScalars));
     S.want(&as, sizeof(AdjScalars));
     S.want(&coef, (size_t)std::max<int64_t>(n, 1) * sizeof(AdjCoef));
-    S.want(&part, std::max(nparts * kSums, (size_t)nb * kFracSums) * sizeof(double));
+    S.want(&part, std::max({nparts * kSums, (size_t)nb * kFracSums, (size_t)nb + kScalarWords}) * sizeof(double));
     if (!S.alloc()) return LAT_ENOMEM;
     Bufs<T> hb = bufs_of<T>(h);
     auto arr = [&](T* base, size_t i) { return base + i * N3; };
@@ -984,47 +984,57 @@ lat_status vjp_impl(lat_handle* h, int64_t n, int64_t ckpt_every, T* fb_user, T*
     };
     rs = forward();
     const lat_status cleared = guard.clear();
+    if (rs == LAT_OK) rs = cleared;
+    const int parN = (int)((s0.step + n) & 1);
+    // The final state is kept and J = <chi^2> formed behind the forward pass, from the
+    // fields where they are, before the host asks for the scalars of the step reached;
+    // one copy brings these and J's partial sums (128^3 FP32, 100 steps: asked for by
+    // themselves they cost 7 to 24 us of 8.4 ms, so 3 to 9).
+    std::vector<double> hp((size_t)nb + kScalarWords);
+    auto finish = [&]() -> lat_status {
+        const T* fN[2];
+        for (int f = 0; f < 2; f++) {
+            fN[f] = n > 0 ? arr(seg, (size_t)(n - clast) * 2 + f) : hb.f[parN][f];
+            LAT_CUDA(cudaMemcpyAsync(fin + f * N3, fN[f], ab, cudaMemcpyDeviceToDevice, st));
+            LAT_CUDA(cudaMemcpyAsync(fin + (2 + f) * N3, hb.p[parN][f], ab, cudaMemcpyDeviceToDevice, st));
+        }
+        LAT_CUDA(cudaMemcpyAsync(fin_sc, h->sc, sizeof(DevScalars), cudaMemcpyDeviceToDevice, st));
+        if (observable != 0) return LAT_OK;
+        LAT_CUDA(cudaMemsetAsync(fb_user, 0, ab, st));
+        LAT_CUDA(cudaMemsetAsync(pb_user, 0, 2 * ab, st));
+        chi2_kernel<T><<<nb, kAdjThreads, 0, st>>>(fN[1], fb_user + N3, (long long)N3, M.inv_sites, part);
+        LAT_CUDA(cudaGetLastError());
+        LAT_CUDA(cudaMemcpyAsync(part + nb, h->sc, sizeof(DevScalars), cudaMemcpyDeviceToDevice, st));
+        LAT_CUDA(cudaMemcpyAsync(hp.data(), part, hp.size() * sizeof(double), cudaMemcpyDeviceToHost, st));
+        LAT_CUDA(cudaStreamSynchronize(st));
+        return LAT_OK;
+    };
+    DevScalars s1;
+    if (rs == LAT_OK) rs = finish();
+    if (rs == LAT_OK && observable == 0) std::memcpy(&s1, hp.data() + nb, sizeof(s1));
+    else LAT_TRY(read_scalars(h, &s1));
     // The fields of the step reached go back into the handle's own set: f_n, or those of
     // an earlier step when its sums were not finite (the steps after it return at once
     // and leave their part of seg unwritten) or a launch was refused. Up to clast the
-    // handle's own arrays hold them. (Reading the scalars here costs nothing that shows:
-    // 128^3 FP32, 100 steps, 8.60 and 8.61 ms without and with.)
-    DevScalars s1;
-    LAT_TRY(read_scalars(h, &s1));
+    // handle's own arrays hold them.
     const int64_t past = s1.step - s0.step - clast;
     for (int f = 0; f < 2 && past > 0; f++)
         LAT_CUDA(cudaMemcpyAsync(hb.f[s1.step & 1][f], arr(seg, (size_t)past * 2 + f), ab, cudaMemcpyDeviceToDevice, st));
-    if (rs == LAT_OK) rs = cleared;
     if (rs == LAT_OK) rs = (lat_status)s1.status;
-    if (rs != LAT_OK) {   // no observable, no reverse sweep: the scratch goes once the copy is done
+    if (rs != LAT_OK) {   // no value, no reverse sweep: the scratch goes once the copy is done
         LAT_CUDA(cudaStreamSynchronize(st));
         return rs;
     }
-    const int parN = (int)((s0.step + n) & 1);
-    for (int f = 0; f < 2; f++) {
-        LAT_CUDA(cudaMemcpyAsync(fin + f * N3, hb.f[parN][f], ab, cudaMemcpyDeviceToDevice, st));
-        LAT_CUDA(cudaMemcpyAsync(fin + (2 + f) * N3, hb.p[parN][f], ab, cudaMemcpyDeviceToDevice, st));
-    }
-    LAT_CUDA(cudaMemcpyAsync(fin_sc, h->sc, sizeof(DevScalars), cudaMemcpyDeviceToDevice, st));
 
     // adjoint of the final state
     AdjScalars a0;
     std::memset(&a0, 0, sizeof(a0));
     if (observable == 0) {
-        LAT_CUDA(cudaMemsetAsync(fb_user, 0, ab, st));
-        LAT_CUDA(cudaMemsetAsync(pb_user, 0, 2 * ab, st));
-        chi2_kernel<T><<<nb, kAdjThreads, 0, st>>>(hb.f[parN][1], fb_user + N3, (long long)N3, M.inv_sites, part);
-        LAT_CUDA(cudaGetLastError());
-        std::vector<double> hp(nb);
-        LAT_CUDA(cudaMemcpyAsync(hp.data(), part, nb * sizeof(double), cudaMemcpyDeviceToHost, st));
-        LAT_CUDA(cudaStreamSynchronize(st));
         double J = 0.0;
         for (int b = 0; b < nb; b++) J += hp[b];
         if (J_out) *J_out = J * M.inv_sites;
     } else if (observable == 1) {
-        DevScalars sF;
-        LAT_CUDA(cudaMemcpyAsync(&sF, fin_sc, sizeof(sF), cudaMemcpyDeviceToHost, st));
-        LAT_CUDA(cudaStreamSynchronize(st));
+        const DevScalars& sF = s1;
         const double at = sF.a - 0.5 * M.dt * sF.ad;
         const double h = M.expansion ? sF.ad / at : 0.0;
         FracConst c;
@@ -1038,7 +1048,7 @@ lat_status vjp_impl(lat_handle* h, int64_t n, int64_t ckpt_every, T* fb_user, T*
         const T *F0 = hb.f[parN][0], *F1 = hb.f[parN][1], *P0 = hb.p[parN][0], *P1 = hb.p[parN][1];
         frac_sums_kernel<T><<<nb, kAdjThreads, 0, st>>>(F0, F1, P0, P1, M.n, c, part);
         LAT_CUDA(cudaGetLastError());
-        std::vector<double> hp((size_t)nb * kFracSums);
+        hp.resize((size_t)nb * kFracSums);
         LAT_CUDA(cudaMemcpyAsync(hp.data(), part, hp.size() * sizeof(double), cudaMemcpyDeviceToHost, st));
         LAT_CUDA(cudaStreamSynchronize(st));
         double S[kFracSums] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
