@@ -552,14 +552,16 @@ lat_status lat_batch_tile_heights(lat_batch* b, int32_t* ty);
 
 /* The launch shape in use (the block shape the paper picks by trial, Sec. II.C
  * and Sec. III, here chosen by lat_batch_tune): out (host) = threads per
- * block, tile-height cap, prefetch depth, blocks. */
+ * block, tile-height cap (0: the whole-row blocks), prefetch depth, blocks. The
+ * first three given to lat_batch_set_shape select the same kernel and blocks. */
 lat_status lat_batch_shape(lat_batch* b, int64_t out[4]);
 
 /* Step with the given shape from now on (the paper fixes its block shape by
  * hand, Sec. II.C): threads per block (32 .. 1024),
- * tile-height cap (1 .. 32) and prefetch depth (1 or 2); the values are those
- * lat_batch_tune sweeps. LAT_EINVAL out of those ranges, LAT_EUNSUPPORTED if
- * some member's tile does not fit the block or the shared memory. Waits for the
+ * tile-height cap (1 .. 32) and prefetch depth (1 or 2), or 256, 0, 2 for the
+ * whole-row blocks; the values are those lat_batch_tune sweeps. LAT_EINVAL for
+ * others, LAT_EUNSUPPORTED if some member's tile does not fit the block or the
+ * shared memory (whole rows: a member that is FP64 or has a side above 128). Waits for the
  * stream first; the member states are not touched. */
 lat_status lat_batch_set_shape(lat_batch* b, int threads, int tycap, int depth);
 

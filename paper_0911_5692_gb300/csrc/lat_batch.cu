@@ -182,10 +182,10 @@ __device__ __forceinline__ void rows_range(const BatchLat<float>& BL, const DevS
 }
 // blocks of eight warps, seven of them with pairs of rows: 14, 28 or 56 rows to a
 // tile by the vectors of a row
-typedef xw::XW<float, 14, 2, false, 32> Rows32;
-typedef xw::XW<float, 28, 2, false, 16> Rows16;
-typedef xw::XW<float, 56, 2, false, 8> Rows8;
-constexpr int kRowThreads = 256, kRowSide = 128;
+constexpr int kRowThreads = 256, kRowSide = 128, kRowDepth = 2;
+typedef xw::XW<float, 14, kRowDepth, false, 32> Rows32;
+typedef xw::XW<float, 28, kRowDepth, false, 16> Rows16;
+typedef xw::XW<float, 56, kRowDepth, false, 8> Rows8;
 static_assert(Rows32::THREADS == kRowThreads && Rows16::THREADS == kRowThreads && Rows8::THREADS == kRowThreads, "");
 constexpr size_t kRowSmem = Rows32::SMEM > Rows16::SMEM ? (Rows32::SMEM > Rows8::SMEM ? Rows32::SMEM : Rows8::SMEM)
                                                         : (Rows16::SMEM > Rows8::SMEM ? Rows16::SMEM : Rows8::SMEM);
@@ -328,7 +328,7 @@ int maxt_of(int threads) { return threads <= 256 ? 256 : threads <= 512 ? 512 : 
 // Shape of one launch.
 struct BatchShape {
     int threads = 0;
-    int tycap = 32;       // largest tile height a member takes
+    int tycap = 32;       // largest tile height a member takes (0: batch_rows_kernel, which cuts its own)
     int depth = 1;        // planes in flight ahead of the one computed
     int maxt = 0;
     bool rows = false;    // batch_rows_kernel
@@ -397,7 +397,8 @@ bool rows_shape(const lat_batch* b, BatchShape* out)
 {
     BatchShape s;
     s.threads = kRowThreads;
-    s.depth = 2;
+    s.tycap = 0;
+    s.depth = kRowDepth;
     s.rows = true;
     s.smem = kRowSmem;
     for (lat_handle* h : b->h) {
@@ -731,7 +732,7 @@ lat_status lat_batch_create(const lat_params* params, int count, void* cuda_stre
         }
         if (tuned.threads) st = configure(b, tuned);
         else {
-            st = configure(b, TunedShape{kRowThreads, 32, 2, true});
+            st = configure(b, TunedShape{kRowThreads, 0, kRowDepth, true});
             for (int t : {256, 512, 384, 640, 768, 1024, 128}) {
                 if (st == LAT_OK) break;
                 st = configure(b, TunedShape{t, 32, 1});
@@ -799,11 +800,12 @@ lat_status lat_batch_tile_heights(lat_batch* b, int32_t* ty)
 
 lat_status lat_batch_set_shape(lat_batch* b, int threads, int tycap, int depth)
 {
-    if (!b || threads < 32 || threads > 1024 || tycap < 1 || tycap > 32 || depth < 1 || depth > 2) return LAT_EINVAL;
+    if (!b) return LAT_EINVAL;
+    // tile cap 0 names the whole-row kernel, with the block and depth it is compiled for
+    const bool rows = tycap == 0 && threads == kRowThreads && depth == kRowDepth;
+    if (!rows && (threads < 32 || threads > 1024 || tycap < 1 || tycap > 32 || depth < 1 || depth > 2)) return LAT_EINVAL;
     LAT_CUDA(cudaStreamSynchronize(b->stream));
-    BatchShape s;
-    if (!shape_for(b, threads, tycap, depth, &s)) return LAT_EUNSUPPORTED;
-    return configure(b, TunedShape{threads, tycap, depth});
+    return configure(b, TunedShape{threads, tycap, depth, rows});
 }
 
 lat_status lat_batch_shape(lat_batch* b, int64_t out[4])

@@ -566,7 +566,9 @@ class Ensemble:
 
     def set_shape(self, threads: int, tile_cap: int, depth: int = 1):
         """Step with this launch shape (threads per block, tile-height cap,
-        prefetch depth) from now on."""
+        prefetch depth) from now on: one that info() reported ("threads",
+        "tile_cap", "depth"; a cap of 0 names the whole-row blocks) or that tune()
+        sweeps."""
         _check(self._L.lat_batch_set_shape(self._h, int(threads), int(tile_cap), int(depth)), "lat_batch_set_shape")
 
     def check_barrier(self, timeout_ns: int = 200_000_000) -> int:
