@@ -319,9 +319,9 @@ lat_status lat_set_kernel(lat_handle* h, int variant, int ty, int zr, int depth)
  * Sec. II.C, keeping 256 computing threads after trying 64, 128 and 256,
  * Sec. III):
  * time `steps` steps (1 <= steps <= 100000, after a warm-up of 32 that also
- * captures the graph) for every kernel shape that can run this lattice --
- * variants 2, 4 and 5 over tile heights and prefetch depths (the 27-point
- * stencil: variants 2 and 5) -- on the lattice's own
+ * captures the graph) for the automatic shape and every kernel shape that can run
+ * this lattice -- variants 2, 4 and 5 over tile heights and prefetch depths (the
+ * 27-point stencil: variants 2 and 5) -- on the lattice's own
  * state, which is saved before and put back after every candidate and at the
  * end; keep the fastest, and remember it for the process per (N, precision,
  * stencil, split storage, expansion), so that handles created later with the

@@ -4,6 +4,7 @@
 #include <cufft.h>
 
 #include <algorithm>
+#include <array>
 #include <cmath>
 #include <cstdlib>
 #include <cstring>
@@ -310,11 +311,13 @@ TuneKey tune_key(const lat_handle* h)
     return TuneKey{h->p.n, h->prec, h->M.stencil, h->M.split, h->M.expansion};
 }
 
-// Candidate shapes for a lattice: every kernel that can run it, over tile
+// Candidate shapes for a lattice: the automatic one, all zero (in FP64 its block count
+// follows from a cost rule and no explicit shape gives it: 40^3 27.2 us per step, the
+// best explicit shape 30.9), then every kernel that can run it, over tile
 // heights and prefetch depths (configure_kernel refuses the ones that do not fit).
 std::vector<TuneShape> tune_candidates(const lat_handle* h)
 {
-    std::vector<TuneShape> c;
+    std::vector<TuneShape> c{{0, 0, 0, 0}};
     if (h->M.stencil == 27) {
         c.push_back({5, 14, 0, 2});
         c.push_back({5, 16, 0, 1});
@@ -523,17 +526,19 @@ lat_status lat_tune(lat_handle* h, int steps, int64_t out[8])
         h->dirty = was_dirty;
         return LAT_OK;
     };
-    const int prev[4] = {h->variant, h->ty, h->zr, h->mcfg.depth};
+    // the launch in use, taken back as it is when the tuning fails
+    const MarchConfig prev = h->mcfg;
+    const int prev_kernel[3] = {h->variant, h->ty, h->zr};
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     if (st == LAT_OK && (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess)) st = LAT_ECUDA;
     TuneShape best{0, 0, 0, 0};
     float best_ms = 0.0f, worst_ms = 0.0f;
-    int tried = 0;
+    std::vector<std::array<int, 5>> tried;   // launches timed: the automatic shape is often one of the explicit ones
     for (const TuneShape& c : tune_candidates(h)) {
         if (st != LAT_OK) break;
         if (configure_kernel(h, c.variant, c.ty, c.zr, c.depth) != LAT_OK) continue;
-        // the geometry the kernel was configured with (an automatic zr, the depth taken)
-        const TuneShape got{h->variant, h->ty, 0, h->mcfg.depth};
+        const std::array<int, 5> launch{h->variant, h->ty, h->mcfg.depth, h->mcfg.blocks, h->mcfg.threads};
+        if (std::find(tried.begin(), tried.end(), launch) != tried.end()) continue;
         if ((st = restore()) != LAT_OK) break;
         // a warm-up that also captures the graph, then the timed steps
         if ((st = lat_evolve(h, kGraphChunk)) != LAT_OK) break;
@@ -547,8 +552,8 @@ lat_status lat_tune(lat_handle* h, int steps, int64_t out[8])
         float ms = 0.0f;
         cudaEventElapsedTime(&ms, e0, e1);
         ms /= (float)steps;
-        tried++;
-        if (!best.variant || ms < best_ms) { best = got; best_ms = ms; }
+        if (tried.empty() || ms < best_ms) { best = c; best_ms = ms; }
+        tried.push_back(launch);
         worst_ms = std::max(worst_ms, ms);
     }
     if (e0) cudaEventDestroy(e0);
@@ -557,19 +562,23 @@ lat_status lat_tune(lat_handle* h, int steps, int64_t out[8])
     if (st == LAT_OK) st = rs;
     if (cudaStreamSynchronize(h->stream) != cudaSuccess && st == LAT_OK) st = LAT_ECUDA;
     cudaFree(save);
-    if (st == LAT_OK && !best.variant) st = LAT_EUNSUPPORTED;
+    if (st == LAT_OK && tried.empty()) st = LAT_EUNSUPPORTED;
     if (st != LAT_OK) {
-        configure_kernel(h, prev[0], prev[1], prev[2], prev[3]);
+        h->mcfg = prev;
+        h->variant = prev_kernel[0];
+        h->ty = prev_kernel[1];
+        h->zr = prev_kernel[2];
+        drop_graph(h);
         return st;
     }
-    LAT_TRY(configure_kernel(h, best.variant, best.ty, 0, best.depth));
+    LAT_TRY(configure_kernel(h, best.variant, best.ty, best.zr, best.depth));
     {
         std::lock_guard<std::mutex> lock(g_tune_mx);
-        g_tuned[tune_key(h)] = TuneShape{best.variant, best.ty, 0, best.depth};
+        g_tuned[tune_key(h)] = best;
     }
     if (out) {
         out[0] = h->variant; out[1] = h->ty; out[2] = h->zr; out[3] = h->mcfg.depth;
-        out[4] = tried;
+        out[4] = (int64_t)tried.size();
         out[5] = (int64_t)std::llround(best_ms * 1e6);   // nanoseconds per step
         out[6] = (int64_t)std::llround(worst_ms * 1e6);
         out[7] = h->mcfg.blocks;
