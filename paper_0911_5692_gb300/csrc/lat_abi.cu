@@ -226,10 +226,14 @@ lat_status configure_kernel(lat_handle* h, int variant, int ty, int zr, int dept
     if (h->M.stencil == 27) {   // the 27-point Laplacian: its own kernels (variants 2 and 5)
         if (variant == 4) return LAT_EUNSUPPORTED;
         MarchConfig cfg;
-        // x tiles one warp wide (sides above 64), but for the two FP64 sides that the
-        // plane ring runs as fast (72^3 182 us per step on both, 80^3 227 against 234;
-        // 68^3 335 against 183, 88^3 329 against 289)
-        const bool ring = h->esize == 8 && n < 88 && n % 8 == 0;
+        // x tiles one warp wide (sides above 64), but for FP64 rows that fill fewer than 22
+        // of an x tile's 32 lanes where the plane ring's tiles of 8 or 16 rows divide the
+        // side: FP64 instructions cost the same whatever their lanes (variant 5 against the
+        // ring, us per step: 72^3, 18 lanes, 181 and 182; 80^3, 20 lanes, 234 and 227; 88^3,
+        // 22 lanes, 288 and 329), and a ring of 4 rows computes five rows for each four
+        // (68^3 179 and 336, 76^3 234 and 454, 84^3 234 and 311).
+        const int q = n / (16 / (int)h->esize), lanes = q / ((q + 31) / 32);
+        const bool ring = h->esize == 8 && lanes < 22 && n % 8 == 0;
         if (variant == 5 || (variant == 0 && !ring)) {
             if (s27w_config(n, (int)h->esize, variant == 0 ? 0 : ty, variant == 0 ? 0 : zr, variant == 0 ? 0 : depth,
                             &cfg) &&
