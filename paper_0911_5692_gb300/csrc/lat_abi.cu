@@ -316,7 +316,7 @@ TuneKey tune_key(const lat_handle* h)
 }
 
 // Candidate shapes for a lattice: the automatic one, all zero (in FP64 its block count
-// follows from a cost rule and no explicit shape gives it: 40^3 27.2 us per step, the
+// follows from a cost rule and no explicit shape gives it: 40^3 24.1 us per step, the
 // best explicit shape 30.9), then every kernel that can run it, over tile
 // heights and prefetch depths (configure_kernel refuses the ones that do not fit).
 std::vector<TuneShape> tune_candidates(const lat_handle* h)
@@ -331,7 +331,7 @@ std::vector<TuneShape> tune_candidates(const lat_handle* h)
     }
     for (int d : {1, 2, 3}) c.push_back({5, 16, 0, d});
     for (int d : {1, 2, 3}) c.push_back({5, 8, 0, d});
-    c.push_back({5, 4, 0, 1});   // FP64: 56^3 45.0 us per step against 47.1 of the automatic shape
+    c.push_back({5, 4, 0, 1});   // FP64
     for (int ty : {32, 16, 8})
         for (int d : {1, 2}) c.push_back({4, ty, 0, d});
     for (int ty : {16, 8, 4, 2})

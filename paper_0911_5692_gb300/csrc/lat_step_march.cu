@@ -240,41 +240,61 @@ bool march_slab_config(int n, int elem_bytes, int nzl, MarchConfig* cfg)
     return false;
 }
 
+// The plane steps of the busiest of `blocks` equal shares of nyt tiles of n planes: the
+// planes it marches, and with them one look-ahead plane for each run (a share that
+// reaches into the next tile starts another).
+void march_busiest(int n, int nyt, long long blocks, int* planes, int* steps)
+{
+    const long long units = (long long)nyt * n;
+    *planes = *steps = 0;
+    for (long long b = 0; b < blocks; b++) {
+        const long long u = b * units / blocks, e = (b + 1) * units / blocks;
+        const int runs = (int)((e - 1) / n - u / n) + 1, p = (int)(e - u);
+        if (p + runs > *steps) {
+            *steps = p + runs;
+            *planes = p;
+        }
+    }
+}
+
 // FP64 tiles and blocks. The step is bound by the FP64 pipes, one per SM sub-
-// partition, 64 cycles per warp instruction: about 32 instructions per two sites
-// that a thread kicks and 16 for the sums of two it owns. A block of ty rows and
-// P planes kicks (ty + 1)(P + 1) rows for its ty P, so tall tiles and long runs
-// cost least, but the busiest sub-partition decides: the tile height and block
-// count are those with the least time there, each plane step costing about 5000
-// cycles (its chain of dependent operations) beside its instructions. 32^3: 64
-// blocks of a plane of 16 rows 24.3 us per step, 128 of 8 rows 17.5; 96^3 150 ->
-// 124; 72^3 88 -> 67; 56^3 55 -> 48.
+// partition, 64 cycles per warp instruction. A plane step of a block of ty rows kicks
+// ty + 1 of them, about 1.9 us per warp of its sub-partition (two sites to a lane, some
+// 32 instructions a site), sums ty, about 1.8 us per warp, and has 1 us that no warp
+// covers; the step lasts as long as the busiest block's plane steps. Taken are the tile
+// height and block count with the least such time, with one block to an SM at most
+// (more are not spread evenly: 289 blocks of 68^3, three to an SM on some, take 86.7 us,
+// 145 65.9): the fewest blocks of which none has more planes than in a full wave, whole
+// chunks of every tile, which start no run in mid share, and the full wave. A block of
+// one warp takes the end of the step without a second one's help (8^3 15.5 us against
+// 14.5). Over sides of 16 to 252 the choice is within 5 % of the best of some 20 shapes,
+// 0.3 % on average. Against the tallest tile in a full wave: 32^3 24.1 -> 17.5 us, 40^3
+// 31.4 -> 24.1, 56^3 56.4 -> 41.9, 68^3 74.5 -> 65.9, 76^3 93.0 -> 77.1, 96^3 148 -> 130,
+// 128^3 254 (the same shape).
 bool march_config_fp64(int n, int depth, MarchConfig* cfg)
 {
-    bool found = false;
     double best = 0.0;
+    bool found = false;
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) return false;
     for (int ty : {16, 8, 4, 2, 1}) {
         MarchConfig c;
         if (!march_geom(n, 8, ty, 0, depth, &c)) continue;
-        const long long units = (long long)c.nyt * n, most = c.blocks;
-        for (int k = 1; k * sms <= std::max<long long>(most, sms); k++) {   // blocks per SM
-            const long long slots = std::min<long long>((long long)k * sms, units);
-            const long long P = (units + slots - 1) / slots, blocks = P >= 8 ? slots : (units + P - 1) / P;
-            const long long per_sm = (blocks + sms - 1) / sms;
-            // warps on the busiest sub-partition (two sites per lane)
-            const double warps = (double)((per_sm * (ty + 1) * (n / 2) + 127) / 128);
-            const double planes = P >= 8 ? (double)units / blocks : (double)P;   // per block
-            const double cost = warps * 128.0 * (32.0 * (planes + 1) + 16.0 * planes) +
-                                5000.0 * per_sm * (planes + 1);
-            if (blocks > most || (found && cost >= best)) continue;
+        const long long units = (long long)c.nyt * n, wave = std::min<long long>({(long long)sms, units, (long long)c.blocks});
+        const long long each = (units + wave - 1) / wave;
+        const double kick = ((ty + 1) * (n / 2) + 31) / 32 / 4.0, sums = (ty * (n / 2) + 31) / 32 / 4.0;   // warps
+        for (long long blocks : {(units + each - 1) / each, wave / c.nyt * c.nyt, wave}) {
+            if (blocks < 1) continue;
+            int planes = 0, steps = 0;
+            march_busiest(n, c.nyt, blocks, &planes, &steps);
+            const double us = steps * (1.0 + 1.9 * kick) + planes * 1.8 * sums + (c.threads > 32 ? 0.0 : 1.0);
+            if (found && us >= best) continue;
             found = true;
-            best = cost;
+            best = us;
             *cfg = c;
             cfg->blocks = (int)blocks;
-            cfg->zr = (int)P;
+            cfg->zr = (int)((units + blocks - 1) / blocks);
             cfg->nzc = (int)((blocks + c.nyt - 1) / c.nyt);
         }
     }
