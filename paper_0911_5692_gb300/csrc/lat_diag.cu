@@ -621,7 +621,8 @@ cudaError_t launch_energies(const Bufs<T>& b, const Model& M, const DevScalars* 
         const int wave = resident_wave((const void*)energies7_kernel<T>, 256, &occ);
         if (wave == 0) return cudaErrorInvalidDevice;
         const long long cols = (long long)(n / V) * (n / 2);
-        const int nzc = balanced_zruns(cols, n, (long long)wave * 256, 0.3);
+        // a plane of a thread is some 14 us of FP64, so small lattices take runs of one
+        const int nzc = balanced_zruns(cols, n, (long long)wave * 256, 0.3, 1);
         blocks = (int)std::min<long long>(wave, (cols * nzc + 255) / 256);
         energies7_kernel<T><<<blocks, 256, 0, st>>>(b, M, sc, partials, nzc);
     }

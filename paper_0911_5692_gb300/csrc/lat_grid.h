@@ -9,13 +9,13 @@ namespace lat {
 
 // Runs per column for `cols` columns of n planes over `threads` threads, where
 // a run of k planes costs k + startup plane-times (the planes loaded before its
-// first one): the count in [1, n/4] that minimises (runs per thread) x (n/runs +
-// startup), the time of the busiest thread.
-inline int balanced_zruns(long long cols, int n, long long threads, double startup)
+// first one): the count in [1, n/least] that minimises (runs per thread) x (n/runs +
+// startup), the time of the busiest thread. least: the shortest run worth starting.
+inline int balanced_zruns(long long cols, int n, long long threads, double startup, int least = 4)
 {
     int best_c = 1;
     double best = 0.0;
-    for (int c = 1; c <= (n / 4 > 1 ? n / 4 : 1); c++) {
+    for (int c = 1; c <= (n / least > 1 ? n / least : 1); c++) {
         const long long per_thread = (cols * c + threads - 1) / threads;
         const double cost = (double)per_thread * ((double)n / c + startup);
         if (c == 1 || cost < best) {
