@@ -547,7 +547,9 @@ lat_status lat_batch_tune(lat_batch* b, int steps);
 
 /* The tile height (y rows per work unit) each member is stepped with:
  * ty (host, one int32 per member, in creation order). The whole-row blocks cut a
- * side into tiles of an uneven number of pairs of rows: 2 for every member. */
+ * side into tiles of uneven height, up to 14, 28 or 56 rows for sides above 64, above
+ * 32 and up to 32; of these the pairs of rows that stay together are given: 2 for every
+ * member. */
 lat_status lat_batch_tile_heights(lat_batch* b, int32_t* ty);
 
 /* The launch shape in use (the block shape the paper picks by trial, Sec. II.C
