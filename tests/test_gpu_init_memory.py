@@ -3,6 +3,7 @@ half spectrum (four arrays of N^3 doubles), and one work area for its transforms
 side with a large prime factor the transforms along x work in two such arrays
 (cuFFT's figure), so six in all; with a work area each it was eight. The free memory
 is read every millisecond beside the call."""
+import gc
 import threading
 import time
 
@@ -20,6 +21,8 @@ def test_transforms_share_one_work_area():
     g = Lattice(lphi4(n, precision=32))
     small = Lattice(lphi4(32, precision=32))
     small.init_fields()       # what the library sets up once is there
+    gc.collect()              # no other test's lattice is freed meanwhile
+    torch.cuda.empty_cache()
     torch.cuda.synchronize()
     before = low = torch.cuda.mem_get_info()[0]
     done = threading.Event()
